@@ -1,0 +1,93 @@
+"""Writes mlkd_fixed_tables.h: the constants of the 64-bit fixed-point
+functions of mlkd_fixed.h.
+
+Every polynomial is evaluated in the form c0 - x (c1 - x (c2 - ...)) with all
+c >= 0: its terms alternate.  The leading coefficients are 64-bit fractions;
+from the first term below 2^-27 on, the rest of the sum is a 32-bit fraction
+scaled by 2^shift.  Coefficients interpolate at the Chebyshev nodes of the
+range, in 50-digit arithmetic, with the degree chosen so that the largest
+error is below 2^-62 (log and sine/cosine use the plain Taylor terms).
+
+    python paper_2004_04071_gb300/csrc/gen_fixed.py > mlkd_fixed_tables.h
+"""
+import mpmath as mp
+
+mp.mp.dps = 50
+TWO64 = mp.mpf(2) ** 64
+
+
+def chebyshev_interpolant(f, hi, deg):
+    """Monomial coefficients (lowest first) of the interpolant of f at the Chebyshev nodes of [0, hi]."""
+    nodes = [hi * (1 + mp.cos(mp.pi * (k + mp.mpf(1) / 2) / (deg + 1))) / 2 for k in range(deg + 1)]
+    V = mp.matrix([[x ** j for j in range(deg + 1)] for x in nodes])
+    c = mp.lu_solve(V, mp.matrix([f(x) for x in nodes]))
+    return [c[j] for j in range(deg + 1)]
+
+
+def series(coef, n0, terms=70):
+    return lambda s: mp.fsum(coef(n) * s ** (n - n0) for n in range(n0, n0 + terms))
+
+
+def near_minimax(f, hi):
+    for deg in range(6, 26):
+        c = chebyshev_interpolant(f, hi, deg)
+        err = max(abs(mp.polyval(list(reversed(c)), hi * i / 400) - f(hi * mp.mpf(i) / 400)) for i in range(401))
+        if err < mp.mpf(2) ** -62:
+            break
+    assert all((-1) ** j * c[j] > 0 for j in range(deg + 1)), "terms do not alternate"
+    return [abs(v) for v in c]
+
+
+def emit(name, c, hi, what):
+    """c: magnitudes of the alternating coefficients, lowest first; x <= hi."""
+    cut = next(j for j in range(len(c)) if c[j] * hi ** j < mp.mpf(2) ** -27)
+    sh = int(mp.floor(-mp.log(c[cut], 2)))
+    lead = [int(mp.nint(min(v * TWO64, TWO64 - 1))) for v in c[:cut]]
+    tail = [int(mp.nint(v * mp.mpf(2) ** (32 + sh))) for v in c[cut:]]
+    while tail[-1] == 0:
+        tail.pop()
+    print("// %s" % what)
+    print("struct %s {" % name)
+    print("    static constexpr int kLead = %d, kTail = %d, kShift = %d;" % (len(lead), len(tail), sh))
+    print("    static constexpr uint64_t lead[kLead] = {")
+    print("        " + ",\n        ".join("0x%016xull" % v for v in lead) + "};")
+    print("    static constexpr uint32_t tail[kTail] = {")
+    print("        " + ", ".join("0x%08xu" % v for v in tail) + "};")
+    print("};")
+
+
+def main():
+    print("// Constants of mlkd_fixed.h, written by gen_fixed.py beside this file.")
+    print("#pragma once\n#include <cstdint>\nnamespace mlkd {\nnamespace fx {")
+    H = series(lambda n: mp.mpf((-1) ** n) / mp.factorial(n), 2)
+    F = series(lambda n: mp.mpf((-1) ** n * (2 - n)) / mp.factorial(n), 3)
+    emit("PolyH", near_minimax(H, mp.mpf(1)), mp.mpf(1), "h(s)/s^2, h(s) = exp(-s) + s - 1, 0 <= s <= 1")
+    emit("PolyF", near_minimax(lambda s: -F(s) if F(mp.mpf(0)) < 0 else F(s), mp.mpf(1)), mp.mpf(1),
+         "f(s)/s^3, f(s) = 2(exp(-s) - 1) + s(exp(-s) + 1), 0 <= s <= 1")
+    hmax = mp.mpf("0.368")
+    emit("PolyW", near_minimax(lambda h: mp.sqrt(2 * H(h)), hmax), hmax,
+         "sqrt(2 (exp(-h) + h - 1))/h, 0 <= h <= exp(-1)")
+    # 2^-f = 1 - f P(f)
+    P = lambda f: (1 - mp.mpf(2) ** -f) / f if f else mp.log(2)
+    emit("PolyE", near_minimax(P, mp.mpf(1)), mp.mpf(1), "(1 - 2^-f)/f, 0 <= f <= 1")
+    # sin z = z (1 - z2 S(z2)), cos z = 1 - z2 C(z2), z2 = z^2 <= (pi/4)^2
+    z2 = (mp.pi / 4) ** 2
+    emit("PolySin", [1 / mp.factorial(2 * k + 3) for k in range(9)], z2, "(1 - sin(z)/z)/z^2 in z^2, |z| <= pi/4")
+    emit("PolyCos", [1 / mp.factorial(2 * k + 2) for k in range(10)], z2, "(1 - cos(z))/z^2 in z^2, |z| <= pi/4")
+    print("constexpr uint64_t kLn2_64 = 0x%016xull;   // ln 2 in 2^-64" % int(mp.nint(mp.log(2) * TWO64)))
+    print("constexpr uint64_t kLn2_58 = 0x%016xull;   // ln 2 in 2^-58" % int(mp.nint(mp.log(2) * mp.mpf(2) ** 58)))
+    print("constexpr uint64_t kLog2e_63 = 0x%016xull; // log2 e in 2^-63" % int(mp.nint(mp.mpf(2) ** 63 / mp.log(2))))
+    print("constexpr uint64_t kTwoPi_61 = 0x%016xull; // 2 pi in 2^-61" % int(mp.nint(2 * mp.pi * mp.mpf(2) ** 61)))
+    # log: reciprocals of the upper ends of 128 intervals of [1/2, 1), and their logarithms
+    C = [(1 << 23) // (129 + j) for j in range(128)]
+    print("// floor(2^15 256/(129 + j)) and ln of that fraction, in 2^-64")
+    print("#define MLKD_LOG_RECIPROCALS \\")
+    print(", \\\n".join("    " + ", ".join("%du" % v for v in C[i:i + 12]) for i in range(0, 128, 12)))
+    print("#define MLKD_LOG_TABLE \\")
+    T = [int(mp.nint(mp.log(mp.mpf(v) / 2 ** 15) * TWO64)) for v in C]
+    print(", \\\n".join("    " + ", ".join("0x%016xull" % v for v in T[i:i + 4]) for i in range(0, 128, 4)))
+    print("}  // namespace fx\n}  // namespace mlkd")
+
+
+if __name__ == "__main__":
+    main()

@@ -592,6 +592,7 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
     __shared__ StartPool<Real> s_start[kWarpsPerBlock];
     __shared__ FinishPool<Real> s_finish[kWarpsPerBlock];
     __shared__ WarpCtx s_ctx[kWarpsPerBlock];
+    init_draw_tables<Real>();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const size_t gw = (size_t)blockIdx.x * kWarpsPerBlock + warp;

@@ -44,6 +44,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     extern __shared__ unsigned int s_hist[];          // [3][nbins]
     __shared__ double s_red[kWarpsPerBlock][kPartialWords];
 
+    init_draw_tables<Real>();
     const int nbins = P.nbins;
     for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x) s_hist[i] = 0u;
     if (nbins > 0) __syncthreads();
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(kThreads)
 coarse_draws_kernel(const __grid_constant__ PairLaunch P, int per_pair, double *nu, double *E,
                     double *chi, int32_t *count)
 {
+    init_draw_tables<Real>();
     const unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= P.n_pairs) return;
     const BgParams<Real> &bp = level_params<Real>(P);

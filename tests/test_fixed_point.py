@@ -1,0 +1,137 @@
+"""The 64-bit fixed-point functions of the FP64 modes (csrc/mlkd_fixed.h),
+compiled for the host and compared with extended-precision library functions.
+
+Bounds, derived from the arithmetic: every function ends in one rounding to
+FP64 (half an ulp) of a fixed-point value whose own error is below 2^-58 (the
+logarithm with whole powers of two, held in units of 2^-58) or 2^-60 (the
+others).  Near u = 1 the logarithm is FP64 arithmetic of five operations,
+each at most half an ulp of a term no larger than the result (2 ulp).
+"""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2004_04071_gb300", "csrc")
+
+SHIM = r"""
+#include "mlkd_fixed.h"
+using namespace mlkd;
+static const uint32_t rc[128] = {MLKD_LOG_RECIPROCALS};
+static const uint64_t ln_[128] = {MLKD_LOG_TABLE};
+struct Tab {
+    uint32_t recip(int j) const { return rc[j]; }
+    uint64_t ln(int j) const { return ln_[j]; }
+};
+template <int B> static fx::Fixed nl(uint64_t n) { return fx::neg_log<B>(n, Tab()); }
+extern "C" void neg_log(int B, const uint64_t *n, int64_t count, double *E, double *r)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        const fx::Fixed f = B == 53 ? nl<53>(n[i]) : nl<24>(n[i]);
+        E[i] = fx::to_double(f.v, f.e);
+        r[i] = fx::sqrt_fixed(f.v, f.e - 1);
+    }
+}
+extern "C" void near_one(const double *w, int64_t count, double *E)
+{
+    for (int64_t i = 0; i < count; ++i) E[i] = fx::log_near_one(w[i]);
+}
+extern "C" void sincos_turn(const uint64_t *p, int64_t count, double *s, double *c)
+{
+    for (int64_t i = 0; i < count; ++i) fx::sincos_turn(p[i], s + i, c + i);
+}
+extern "C" void roots(const double *x, int64_t count, double *s, double *r)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        s[i] = fx::sqrt_normal(x[i]);
+        r[i] = fx::rsqrt_normal(x[i]);
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def fx(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fixed")
+    src, so = str(d / "shim.cpp"), str(d / "shim.so")
+    with open(src, "w") as fh:
+        fh.write(SHIM)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
+    return ctypes.CDLL(so)
+
+
+def call(f, *args):
+    f.restype = None
+    f(*[ctypes.c_int64(a) if isinstance(a, int) else a.ctypes.data_as(ctypes.c_void_p) for a in args])
+
+
+def ulp(x):
+    return np.spacing(np.abs(x).astype(np.float64)).astype(np.longdouble)
+
+
+@pytest.mark.parametrize("B", [53, 24])
+def test_logarithm_and_radius(fx, B):
+    """Every power of two and its neighbours, both ends of every table
+    interval, the smallest uniform, the largest below the near-one branch, and
+    random ones."""
+    rng = np.random.default_rng(B)
+    top = 1 << B
+    n = [1, 2, 3, top - (1 << (B - 12)), top - (1 << (B - 12)) - 1]
+    for k in range(B):
+        n += [(1 << k) - 1, 1 << k, (1 << k) + 1]
+    for j in range(129):
+        edge = (128 + j) << (B - 8)
+        n += [edge - 1, edge, edge + 1]
+    n += [int(v) for v in rng.integers(1, top, 20000)] + [int(v) >> int(s) for v, s in
+                                                         zip(rng.integers(top // 2, top, 5000), rng.integers(0, B - 1, 5000))]
+    n = np.array([v for v in n if 1 <= v <= top - (1 << (B - 12))], np.uint64)
+    E, r = np.zeros(len(n)), np.zeros(len(n))
+    fx.neg_log.restype = None
+    fx.neg_log(B, n.ctypes.data_as(ctypes.c_void_p), ctypes.c_int64(len(n)), E.ctypes.data_as(ctypes.c_void_p),
+               r.ctypes.data_as(ctypes.c_void_p))
+    exact = -np.log(n.astype(np.longdouble) / np.longdouble(top))
+    assert np.all(np.abs(E - exact) <= ulp(E) + np.longdouble(2.0) ** -58)
+    root = np.sqrt(2 * exact)
+    assert np.all(np.abs(r - root) <= ulp(r) + np.longdouble(2.0) ** -58 / root)
+
+
+def test_logarithm_near_one(fx):
+    w = np.concatenate([[0.0, 2.0**-53, 2.0**-24, 2.0**-12 - 2.0**-53], 2.0 ** -np.random.default_rng(1).uniform(12.01, 52, 2000)])
+    E = np.zeros(len(w))
+    call(fx.near_one, w, len(w), E)
+    exact = -np.log1p(-w.astype(np.longdouble))
+    assert E[0] == 0.0
+    assert np.all(np.abs(E - exact) <= 2 * ulp(exact))
+
+
+def test_sine_and_cosine(fx):
+    """All octant boundaries and their neighbours, the axes, random phases."""
+    rng = np.random.default_rng(3)
+    p = [(k << 60) + d for k in range(16) for d in (-2048, -1, 0, 1, 2048)]
+    p = np.array([v % (1 << 64) for v in p] + [int(v) << 11 for v in rng.integers(0, 1 << 53, 20000)]
+                 + [int(v) << 40 for v in rng.integers(0, 1 << 24, 20000)], np.uint64)
+    s, c = np.zeros(len(p)), np.zeros(len(p))
+    call(fx.sincos_turn, p, len(p), s, c)
+    # the residual from the nearest quarter turn is exact
+    k = ((p >> np.uint64(61)) + np.uint64(1)) >> np.uint64(1)
+    z = (p - (k << np.uint64(62))).view(np.int64).astype(np.longdouble) * (8 * np.arctan(np.longdouble(1))) / np.longdouble(2) ** 64
+    q = (k & np.uint64(3)).astype(int)
+    es = np.choose(q, [np.sin(z), np.cos(z), -np.sin(z), -np.cos(z)])
+    ec = np.choose(q, [np.cos(z), -np.sin(z), -np.cos(z), np.sin(z)])
+    bound = np.longdouble(2.0) ** -54 + np.longdouble(2.0) ** -60
+    assert np.all(np.abs(s - es) <= bound) and np.all(np.abs(c - ec) <= bound)
+    assert s[2] == 0.0 and c[2] == 1.0
+
+
+def test_square_roots(fx):
+    rng = np.random.default_rng(4)
+    x = np.concatenate([[1.0, 2.0, 4.0, 0.25, np.nextafter(1.0, 0), np.nextafter(4.0, 0), np.nextafter(1.0, 2), 2.0**-1022, 1.7e308],
+                        2.0 ** rng.uniform(-1000, 1000, 20000)])
+    s, r = np.zeros(len(x)), np.zeros(len(x))
+    call(fx.roots, x, len(x), s, r)
+    xl = x.astype(np.longdouble)
+    assert np.all(np.abs(s - np.sqrt(xl)) <= 0.6 * ulp(s))
+    assert np.all(np.abs(r - 1 / np.sqrt(xl)) <= 0.6 * ulp(r))
