@@ -3,7 +3,7 @@ functions of mlkd_fixed.h.
 
 Every polynomial is evaluated in the form c0 - x (c1 - x (c2 - ...)) with all
 c >= 0: its terms alternate.  The leading coefficients are 64-bit fractions;
-from the first term below 2^-27 on, the rest of the sum is a 32-bit fraction
+from the first term below 2^-29 on, the rest of the sum is a 32-bit fraction
 scaled by 2^shift.  Coefficients interpolate at the Chebyshev nodes of the
 range, in 50-digit arithmetic, with the degree chosen so that the largest
 error is below 2^-62 (log and sine/cosine use the plain Taylor terms).
@@ -40,7 +40,7 @@ def near_minimax(f, hi):
 
 def emit(name, c, hi, what):
     """c: magnitudes of the alternating coefficients, lowest first; x <= hi."""
-    cut = next(j for j in range(len(c)) if c[j] * hi ** j < mp.mpf(2) ** -27)
+    cut = next(j for j in range(len(c)) if c[j] * hi ** j < mp.mpf(2) ** -29)
     sh = int(mp.floor(-mp.log(c[cut], 2)))
     lead = [int(mp.nint(min(v * TWO64, TWO64 - 1))) for v in c[:cut]]
     tail = [int(mp.nint(v * mp.mpf(2) ** (32 + sh))) for v in c[cut:]]

@@ -41,6 +41,8 @@ MLKD_HD int clz64(uint64_t v)
 #endif
 }
 
+MLKD_HD int max_int(int a, int b) { return a > b ? a : b; }
+
 MLKD_HD uint64_t bits_of(double x)
 {
 #ifdef __CUDA_ARCH__
@@ -91,7 +93,7 @@ MLKD_HD uint64_t mul64x32(uint64_t a, uint32_t b)
 MLKD_HD uint32_t mul32(uint32_t a, uint32_t b) { return (uint32_t)((uint64_t)a * b >> 32); }
 
 // c0 - x (c1 - x (c2 - ...)) for a fraction x: the tail of the sum (terms
-// below 2^-27) in 32 bits, the rest in 64
+// below 2^-29) in 32 bits, the rest in 64
 template <typename P, int I> MLKD_HD uint32_t poly_tail(uint32_t x)
 {
     constexpr uint32_t c = P::tail[I];
@@ -274,13 +276,12 @@ MLKD_HD void sincos_turn(uint64_t phase, double *sn, double *cs)
 MLKD_HD uint64_t exp_neg(double x)
 {
     const uint64_t b = bits_of(x);
-    const int ex = (int)(b >> 52) - 1023;                     // x in [2^ex, 2^(ex + 1))
-    const uint64_t m = (b << 11) | 0x8000000000000000ull;
-    const uint64_t x58 = m >> ((5 - ex) & 63);                // x 2^58 for x < 64
-    const uint64_t y = mul64(x58, kLog2e_63);                 // x log2 e 2^57
-    const uint64_t f = y << 7;
+    const int ex = max_int((int)(b >> 52) - 1023, -2);        // x = m 2^(ex - 63)
+    const uint64_t m = ((b << 11) | 0x8000000000000000ull) >> ((ex + 1023 - (int)(b >> 52)) & 63);
+    const uint64_t y = mul64(m, kLog2e_63);                   // x log2 e 2^(62 - ex)
+    const uint64_t f = y << ((ex + 2) & 63);
     const uint64_t p = ~mul64(f, poly<PolyE>(f));
-    return x < 44.0 ? p >> ((int)(y >> 57) & 63) : 0u;
+    return (uint32_t)(b >> 32) < 0x40460000u ? p >> (int)(((y >> 1) >> ((61 - ex) & 63)) & 63u) : 0u;    // 44.0
 }
 
 }  // namespace fx

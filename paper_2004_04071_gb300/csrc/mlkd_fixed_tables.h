@@ -5,7 +5,7 @@ namespace mlkd {
 namespace fx {
 // h(s)/s^2, h(s) = exp(-s) + s - 1, 0 <= s <= 1
 struct PolyH {
-    static constexpr int kLead = 10, kTail = 3, kShift = 28;
+    static constexpr int kLead = 11, kTail = 2, kShift = 32;
     static constexpr uint64_t lead[kLead] = {
         0x8000000000000000ull,
         0x2aaaaaaaaaaaaa4cull,
@@ -16,9 +16,10 @@ struct PolyH {
         0x0001a019ff3938fdull,
         0x00002e3bc0383aecull,
         0x0000049f85a3e4efull,
-        0x0000006b852e0d27ull};
+        0x0000006b852e0d27ull,
+        0x00000008e48f9e46ull};
     static constexpr uint32_t tail[kTail] = {
-        0x8e48f9e4u, 0x0a4dbf71u, 0x008364b3u};
+        0xa4dbf70au, 0x08364b2au};
 };
 // f(s)/s^3, f(s) = 2(exp(-s) - 1) + s(exp(-s) + 1), 0 <= s <= 1
 struct PolyF {
@@ -39,20 +40,21 @@ struct PolyF {
 };
 // sqrt(2 (exp(-h) + h - 1))/h, 0 <= h <= exp(-1)
 struct PolyW {
-    static constexpr int kLead = 6, kTail = 4, kShift = 18;
+    static constexpr int kLead = 7, kTail = 3, kShift = 22;
     static constexpr uint64_t lead[kLead] = {
         0xffffffffffffffffull,
         0x2aaaaaaaaaaaaa9bull,
         0x071c71c71c71c174ull,
         0x00f2b9d6480e6752ull,
         0x001948b0fcc96afaull,
-        0x00020bfad21b8142ull};
+        0x00020bfad21b8142ull,
+        0x000021e78ee38e7bull};
     static constexpr uint32_t tail[kTail] = {
-        0x879e3b8eu, 0x0837f244u, 0x0098fe4du, 0x000a4137u};
+        0x837f243au, 0x098fe4d6u, 0x00a41374u};
 };
 // (1 - 2^-f)/f, 0 <= f <= 1
 struct PolyE {
-    static constexpr int kLead = 9, kTail = 3, kShift = 27;
+    static constexpr int kLead = 10, kTail = 2, kShift = 31;
     static constexpr uint64_t lead[kLead] = {
         0xb17217f7d1cf79aaull,
         0x3d7f7bff058b1acbull,
@@ -62,20 +64,22 @@ struct PolyE {
         0x000a184895de347aull,
         0x0000ffe5f74da630ull,
         0x0000162bf1b6bc61ull,
-        0x000001b50af3e60dull};
+        0x000001b50af3e60dull,
+        0x0000001e31028c6aull};
     static constexpr uint32_t tail[kTail] = {
-        0xf1881463u, 0x0eadd7ccu, 0x00a46768u};
+        0xeadd7cbeu, 0x0a46767du};
 };
 // (1 - sin(z)/z)/z^2 in z^2, |z| <= pi/4
 struct PolySin {
-    static constexpr int kLead = 4, kTail = 5, kShift = 25;
+    static constexpr int kLead = 5, kTail = 4, kShift = 32;
     static constexpr uint64_t lead[kLead] = {
         0x2aaaaaaaaaaaaaabull,
         0x0222222222222222ull,
         0x000d00d00d00d00dull,
-        0x00002e3bc74aad8eull};
+        0x00002e3bc74aad8eull,
+        0x0000006b99159fd5ull};
     static constexpr uint32_t tail[kTail] = {
-        0xd7322b40u, 0x01612461u, 0x0001ae7fu, 0x00000195u, 0x00000001u};
+        0xb092309du, 0x00d73f9fu, 0x0000ca96u, 0x00000098u};
 };
 // (1 - cos(z))/z^2 in z^2, |z| <= pi/4
 struct PolyCos {

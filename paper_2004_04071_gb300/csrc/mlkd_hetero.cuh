@@ -244,8 +244,14 @@ __device__ __forceinline__ bool het_pair_event(HetPairState<Real> &st, const Het
     // Sec. 3.2 aggregation: beta of this phase (rate Rloc), then alpha of
     // the new phase if the window goes on
     const Real invR = Arith<Real>::div_(Real(1), Rloc);
-    const Real hp = hs < Real(1) ? hs * hs * A::h_series(hs) : A::exp_(-hs) + hs - Real(1);
-    const Real beta = A::sqrt_pos_(Real(2) * hp) * invR;          // eq. weights-beta, sigma = 1
+    Real beta;                                                    // eq. weights-beta, sigma = 1
+    if constexpr (std::is_same<Real, double>::value) {
+        double b2;
+        beta = Background<double>{}.beta_hat(hs, b2) * invR;
+    } else {
+        const Real hp = hs < Real(1) ? hs * hs * A::h_series(hs) : A::exp_(-hs) + hs - Real(1);
+        beta = A::sqrt_pos_(Real(2) * hp) * invR;
+    }
     if (st.fresh) {
         st.chi_first = d.chi;
         st.fresh = false;

@@ -134,12 +134,13 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
     if (coupled) {
         // Sec. 3.2 aggregation, streamed: this phase's chi with beta, and the
         // new phase's nu with alpha if it collides inside the coarse step.
-        const Real bh2 = bg.beta_hat_sq(hs);
+        Real bh2;
+        const Real bh = bg.beta_hat(hs, bh2);
         if (st.fresh) {
             st.chi_first = d.chi;
             st.fresh = false;
         }
-        st.num += A::sqrt_pos_(bh2) * d.chi;
+        st.num += bh * d.chi;
         st.den += bh2;
         if (st.qf < (Real)(st.Ec - st.i_f)) {
             const Real ah = st.qf * bg.Rdt + om;                  // R tau' = R tau + R zeta

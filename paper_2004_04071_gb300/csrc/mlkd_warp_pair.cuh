@@ -113,9 +113,10 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             if (lane == 0) Kp = L.divM(st.Ec) - 1;             // coarse step of the carried collision
             const bool trig = valid && Kn != Kp;
             const unsigned tmask = __ballot_sync(kFullMask, trig);
-            const Real bh2 = valid ? bg.beta_hat_sq(hs) : Real(0);
-            Real cn = valid ? A::sqrt_pos_(bh2) * d.chi : Real(0);
-            Real cd = bh2;
+            Real bh2;
+            const Real bh = bg.beta_hat(hs, bh2);
+            Real cn = valid ? bh * d.chi : Real(0);
+            Real cd = valid ? bh2 : Real(0);
             if (valid && !trig) {
                 const Real ah = qn * bg.Rdt + om;              // R tau' = R tau + R zeta
                 cn += ah * d.nu;

@@ -50,6 +50,16 @@ extern "C" void roots(const double *x, int64_t count, double *s, double *r)
         r[i] = fx::rsqrt_normal(x[i]);
     }
 }
+extern "C" void kd(const double *s, int64_t count, double *H, double *F, double *W, double *e)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        const uint64_t x = fx::fraction(s[i] < 1.0 ? s[i] : 0.0);
+        H[i] = fx::to_double_62(fx::poly<fx::PolyH>(x), 64);
+        F[i] = fx::to_double(fx::poly<fx::PolyF>(x), 64);
+        W[i] = fx::to_double_62(fx::poly<fx::PolyW>(fx::fraction(s[i] < 1.0 ? s[i] * 0.36787944117144233 : 0.0)) >> 1, 63);
+        e[i] = s[i] >= 0.0625 ? fx::to_double(fx::exp_neg(s[i]), 64) : 0.0;
+    }
+}
 """
 
 
@@ -135,3 +145,35 @@ def test_square_roots(fx):
     xl = x.astype(np.longdouble)
     assert np.all(np.abs(s - np.sqrt(xl)) <= 0.6 * ulp(s))
     assert np.all(np.abs(r - 1 / np.sqrt(xl)) <= 0.6 * ulp(r))
+
+
+def taylor(coef, n0, s, terms=30):
+    """sum_{n >= n0} coef(n) s^(n - n0), smallest terms first."""
+    out = np.zeros_like(s)
+    for n in range(n0 + terms, n0 - 1, -1):
+        out = out * s + coef(n)
+    return out
+
+
+def test_coefficient_polynomials_and_exponential(fx):
+    """H = h/s^2, F = f/s^3, W = sqrt(2 h)/h-argument and e^-s over their
+    ranges, the ends and tiny arguments among them (e^-s to 2^-58
+    absolute)."""
+    rng = np.random.default_rng(5)
+    s = np.concatenate([[0.0, 2.0**-1000, 2.0**-64, 2.0**-63, 1e-5, 0.5, np.nextafter(1.0, 0)], rng.uniform(0, 1, 20000),
+                        2.0 ** -rng.uniform(1, 60, 3000), [1.0, 1.0000001, 43.999999, 44.0, 63.9, 64.0, 1e9],
+                        rng.uniform(1, 46, 20000)])
+    H, F, W, e = (np.zeros(len(s)) for _ in range(4))
+    call(fx.kd, s, len(s), H, F, W, e)
+    small = s < 1
+    fact = np.cumprod(np.concatenate([[1], np.arange(1, 40)]).astype(np.longdouble))
+    t = s[small].astype(np.longdouble)
+    h = lambda n: (-1.0) ** n / fact[n]                                # noqa: E731
+    f = lambda n: (-1.0) ** n * (2 - n) / fact[n]                      # noqa: E731
+    eps = np.longdouble(2.0) ** -60
+    for got, exact in ((H[small], taylor(h, 2, t)), (F[small], taylor(f, 3, t)),
+                       (W[small], np.sqrt(2 * taylor(h, 2, (s[small] * 0.36787944117144233).astype(np.longdouble))))):
+        assert np.all(np.abs(got - exact) <= 0.5 * ulp(exact) + eps)
+    big = s >= 0.0625
+    exact = np.exp(-s[big].astype(np.longdouble))
+    assert np.all(np.abs(e[big] - exact) <= 0.5 * ulp(exact) + np.longdouble(2.0) ** -58)
