@@ -659,6 +659,8 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
             L.bg.dt = bp.dt;
             L.bg.Rdt = bp.Rdt;
             L.bg.inv_Rdt = bp.inv_Rdt;
+            L.bg.c = bp.c;
+            L.bg.c_lo = bp.c_lo;
             L.n = D->n_level[level];
             L.M = D->M_level[level];
             L.divM.init(L.M);
@@ -821,10 +823,12 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
                 pair_start_values<Real, RECIPE>(x0, v0, q0, pr, L, B.keys);
             }
         }
-        const bool dead = have && !(q0 < (Real)L.n);
+        bool dead;
+        if constexpr (PHYS == 1) dead = have && !(q0 < (Real)L.n);
+        else dead = have && !collides_before_T(L, q0);
         Real xT = Real(0);
         if (dead) {
-            xT = x0 + v0 * ((Real)L.n * L.bg.dt);          // pair_drift from t = 0
+            xT = straight_to_T<Real, PHYS>(x0, v0, L);
             dbg_record(pr, xT, xT, 0u, 0u);
         }
         fp_push(dead, xT, coupled ? xT : Real(0), 0u, 0u);

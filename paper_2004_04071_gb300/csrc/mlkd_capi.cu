@@ -207,6 +207,8 @@ void fill_launch(const mlkd_problem *p, const Derived &d, int j, uint64_t first,
     b.dt = P->dt;
     b.Rdt = P->R * P->dt;
     b.inv_Rdt = 1.0 / (P->R * P->dt);
+    b.c = P->sigma / P->R;
+    b.c_lo = std::fma(-b.c, P->R, P->sigma) / P->R;
     b.lo = P->lo;
     b.hi = P->hi;
     b.inv_h = 1.0 / P->h;
@@ -219,6 +221,8 @@ void fill_launch(const mlkd_problem *p, const Derived &d, int j, uint64_t first,
     f.dt = (float)b.dt;
     f.Rdt = (float)b.Rdt;
     f.inv_Rdt = (float)b.inv_Rdt;
+    f.c = (float)b.c;
+    f.c_lo = 0.0f;
     f.lo = (float)b.lo;
     f.hi = (float)b.hi;
     f.inv_h = (float)b.inv_h;

@@ -136,6 +136,57 @@ MLKD_HD uint64_t fraction(double x)
     return sh < 64 ? m >> sh : 0u;
 }
 
+// n as a double, n >= 1
+MLKD_HD double from_u32(uint32_t n)
+{
+#ifdef __CUDA_ARCH__
+    const int lz = __clz((int)n);
+#else
+    const int lz = __builtin_clz(n);
+#endif
+    const uint32_t m = n << lz;
+    return from_bits(((uint64_t)(uint32_t)((1023 + 31 - 1 - lz) << 20) << 32) + ((uint64_t)m << 21));
+}
+
+// A flight q >= 0 in steps: whole = floor(q) (at most 2^31 - 1) and
+// left = (whole + 1 - q) 2^64, the part of the collision's step that is left
+// (2^64 - 1 for a whole step)
+struct Flight {
+    int whole;
+    uint64_t left;
+};
+MLKD_HD Flight split_flight(double q)
+{
+    const uint64_t b = bits_of(q);
+    const int ex = (int)(b >> 52) - 1023;
+    const uint64_t m = (b << 11) | 0x8000000000000000ull;     // q = m 2^(ex - 63)
+    Flight f;
+    uint64_t frac;
+    if (ex < 0) {
+        f.whole = 0;
+        frac = ex > -64 ? m >> ((-1 - ex) & 63) : 0u;
+    } else {
+        f.whole = ex < 31 ? (int)(uint32_t)(m >> ((63 - ex) & 63)) : 0x7fffffff;
+        frac = ex < 63 ? m << ((ex + 1) & 63) : 0u;
+    }
+    f.left = frac ? 0u - frac : ~(uint64_t)0;
+    return f;
+}
+
+// steps + left 2^-64 as a double (steps >= 0)
+MLKD_HD double steps_left(int steps, uint64_t left)
+{
+    if (steps == 0) return to_double(left, 64);
+#ifdef __CUDA_ARCH__
+    const int lz = __clz(steps);
+#else
+    const int lz = __builtin_clz((uint32_t)steps);
+#endif
+    // the leading bit of the 96-bit number comes to bit 63; lz >= 1
+    const uint64_t v = ((uint64_t)(uint32_t)steps << (32 + lz)) | (left >> (32 - lz));
+    return from_bits(((uint64_t)(1023 + 31 - 1 - lz) << 52) + (v >> 11) + ((v >> 10) & 1u));
+}
+
 // ---------------------------------------------------------------------------
 // -ln u = v 2^-e for the uniform u = n 2^-B, 1 <= n <= 2^B.  n is normalised
 // to x in [1/2, 1); with the reciprocal c of the upper end of x's interval

@@ -58,6 +58,7 @@ template <typename Real> struct BgParams {
     Real R, invR, mu, sigma;
     Real two_c2;      // 2 sigma^2 / R^2
     Real dt, Rdt, inv_Rdt;
+    Real c, c_lo;     // sigma / R, and the rest of its rounding (FP64)
     Real lo, hi, inv_h;
 };
 

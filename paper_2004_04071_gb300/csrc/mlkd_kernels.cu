@@ -59,6 +59,8 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     L.bg.dt = bp.dt;
     L.bg.Rdt = bp.Rdt;
     L.bg.inv_Rdt = bp.inv_Rdt;
+    L.bg.c = bp.c;
+    L.bg.c_lo = bp.c_lo;
     L.n = P.n;
     L.M = P.M;
     L.divM.init(P.M);
@@ -155,10 +157,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
                         none = het_pair_start<Real, RECIPE>(st, cand, H, P.keys, COUPLED);
                     } else {
                         none = pair_start<Real, CPL, RECIPE>(st, cand, L, P.keys, COUPLED);
-                        if (P.init == 2) {
-                            st.xf = (Real)P.x0;
-                            st.xc = st.xf;
-                        }
+                        if (P.init == 2) set_start(st, (Real)P.x0);
                     }
                     if (none)
                         done = true;
@@ -302,6 +301,8 @@ coarse_draws_kernel(const __grid_constant__ PairLaunch P, int per_pair, double *
     L.bg.dt = bp.dt;
     L.bg.Rdt = bp.Rdt;
     L.bg.inv_Rdt = bp.inv_Rdt;
+    L.bg.c = bp.c;
+    L.bg.c_lo = bp.c_lo;
     L.n = P.n;
     L.M = P.M;
     L.divM.init(P.M);

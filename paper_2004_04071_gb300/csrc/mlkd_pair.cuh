@@ -24,7 +24,21 @@ namespace mlkd {
 // NoTrace compiles to nothing.
 struct NoTrace {};
 
-template <typename Real> struct PairState {
+// FP64 state is dimensionless: with velocities mu + sigma nu, the position
+// is x = x_0 + mu t + (sigma/R) y, a kinetic phase of optical length E moves y by
+// nu E, and no coefficient of the background is left in the KD step but R dt.
+// xf, xc hold y and vf, vc hold nu.  One pair per lane keeps a flight as its
+// optical length and its split into whole steps and the rest of the
+// collision's step; one pair per warp keeps it as qf, qc.
+template <typename Real> struct FlightState {};
+template <> struct FlightState<double> {
+    double x0;                  // initial position
+    double of, oc;              // optical lengths E of the fine and coarse flights
+    uint64_t left_f, left_c;    // 2^64 (whole + 1 - flight in steps)
+    int whole_f, whole_c;
+};
+
+template <typename Real> struct PairState : FlightState<Real> {
     Real xf, vf, qf;            // fine path: position, velocity, flight (fine units)
     Real xc, vc, qc;            // coarse path
     Real num, den, chi_first;   // streamed eq. chi-update of the open coarse window
@@ -56,9 +70,31 @@ __device__ __forceinline__ int next_coarse_end(const LevelCtx<Real> &L, int base
 template <typename Real, int CPL>
 __device__ __forceinline__ bool pair_is_coupled(bool runtime) { return CPL == 2 ? runtime : CPL == 1; }
 
+// Position x at T from the FP64 pair state.  c = sigma/R enters as the sum of
+// two numbers: rounded to one it would shift every pair's x alike.
+__device__ __forceinline__ double position_at_T(const LevelCtx<double> &L, double x0, double y)
+{
+    return fma(L.bg.c, y, fma(L.bg.c_lo, y, fma(L.bg.mu, (double)L.n * L.bg.dt, x0)));
+}
+
+// A pair's first flight, drawn as E (FP64) or in fine steps (FP32): in fine
+// steps, and whether its collision lies before T.
+template <typename Real> __device__ __forceinline__ Real first_flight(const LevelCtx<Real> &L, Real q0)
+{
+    if constexpr (std::is_same<Real, double>::value) return q0 * L.bg.inv_Rdt;
+    else return q0;
+}
+template <typename Real> __device__ __forceinline__ bool collides_before_T(const LevelCtx<Real> &L, Real q0)
+{
+    if constexpr (std::is_same<Real, double>::value)
+        return fx::split_flight(first_flight(L, q0)).whole < L.n;
+    else
+        return q0 < (Real)L.n;
+}
+
 // Alg. 1 / Alg. 2 initialisation values of pair p: x_0, v_0 and the first
-// flight in fine-step units (nu_0, E_0 and the initial-position uniform of
-// Philox block 0), shared by both paths.
+// flight (nu_0, E_0 and the initial-position uniform of Philox block 0),
+// shared by both paths; FP64: nu_0 and E_0.
 template <typename Real, int RECIPE = 0>
 __device__ __forceinline__ void pair_start_values(Real &x0, Real &v0, Real &q0, unsigned long long p,
                                                   const LevelCtx<Real> &L, const PhiloxKeys &keys)
@@ -66,8 +102,24 @@ __device__ __forceinline__ void pair_start_values(Real &x0, Real &v0, Real &q0, 
     const Draw<Real> d0 = draw_r<Real, RECIPE>(0u, (uint32_t)p, L.word2 ^ (uint32_t)(p >> 32),
                                                L.request, keys);
     x0 = L.init ? cosine_inverse<Real>(d0.u4) : Real(0);
-    v0 = L.bg.mu + L.bg.sigma * d0.nu;
-    q0 = d0.E * L.bg.inv_Rdt;
+    if constexpr (std::is_same<Real, double>::value) {
+        v0 = d0.nu;
+        q0 = d0.E;
+    } else {
+        v0 = L.bg.mu + L.bg.sigma * d0.nu;
+        q0 = d0.E * L.bg.inv_Rdt;
+    }
+}
+
+// Both paths of the pair start at x0.
+template <typename Real> __device__ __forceinline__ void set_start(PairState<Real> &st, Real x0)
+{
+    if constexpr (std::is_same<Real, double>::value) {
+        st.x0 = x0;
+        st.xf = st.xc = 0.0;
+    } else {
+        st.xf = st.xc = x0;
+    }
 }
 
 // The state of pair p at t = 0 from its initialisation values.  Returns true
@@ -79,23 +131,33 @@ __device__ __forceinline__ bool pair_init(PairState<Real> &st, unsigned long lon
     const bool coupled = pair_is_coupled<Real, CPL>(coupled_rt);
     st.pair_lo = (uint32_t)p;
     st.word2 = L.word2 ^ (uint32_t)(p >> 32);
-    st.xf = x0;
+    const Real qf = first_flight(L, q0);
+    set_start(st, x0);
     st.vf = v0;
-    st.qf = q0;
+    st.qf = qf;
     st.i_f = 0;
     st.k = 0;
     st.evc = 0;
+    int whole;
+    if constexpr (std::is_same<Real, double>::value) {
+        const fx::Flight fl = fx::split_flight(qf);
+        whole = fl.whole;
+        st.of = st.oc = q0;
+        st.whole_f = st.whole_c = fl.whole;
+        st.left_f = st.left_c = fl.left;
+    } else {
+        whole = (int)qf;
+    }
     if (coupled) {
-        st.xc = x0;
         st.vc = v0;
-        st.qc = q0;
+        st.qc = qf;
         st.ic = 0;
         st.num = Real(0);
         st.den = Real(0);
         st.fresh = true;
-        if (q0 < (Real)L.n) st.Ec = next_coarse_end(L, 0, (int)q0);
+        if (qf < (Real)L.n) st.Ec = next_coarse_end(L, 0, whole);
     }
-    return !(q0 < (Real)L.n);
+    return !(qf < (Real)L.n);
 }
 
 // Returns true if the pair has no collision before T (already finished).
@@ -109,12 +171,83 @@ __device__ __forceinline__ bool pair_start(PairState<Real> &st, unsigned long lo
     return pair_init<Real, CPL>(st, p, x0, v0, q0, L, coupled_rt);
 }
 
+// One fine event of the FP64 state; returns true when the pair has reached T.
+// The FP64 pipe bounds it (two operations per clock and SM), so everything
+// that can be is integer: draws, coefficients and roots in fixed point, step
+// counts and window tests on the whole part of a flight, conversions by
+// moving bits.  19 FP64 operations are left per fine event and 12 per coarse
+// one, against about 45 and 27 with positions in x and times in FP64: level 8
+// of the periodic problem, 131 071 pairs, 2.41 -> 1.86 ms.
+template <int CPL, int RECIPE, typename Trace>
+__device__ __forceinline__ bool pair_event_fp64(PairState<double> &st, const LevelCtx<double> &L,
+                                                const PhiloxKeys &keys, bool coupled_rt, Trace *tr)
+{
+    typedef Arith<double> A;
+    const bool coupled = pair_is_coupled<double, CPL>(coupled_rt);
+    const Background<double> &bg = L.bg;
+    const Draw<double> d = draw_r<double, RECIPE>(st.k + 1u, st.pair_lo, st.word2, L.request, keys);
+    const double s = bg.Rdt * fx::to_double(st.left_f, 64);     // R theta (eq. diffusive-time)
+    const double nu2 = d.nu * d.nu;
+    double D, hs, om;
+    Background<double>::kd_unit(s, nu2, D, hs, om);
+    // eq. position-update: nu_k E_k, then nu_{k+1} (1 - e^{-s}) + D chi_k; one
+    // rounding at the size of y
+    st.xf += fma(st.vf, st.of, fma(D, d.chi, d.nu * om));
+    st.i_f += st.whole_f + 1;                                   // eq. time-update
+    st.vf = d.nu;
+    st.of = d.E;
+    const fx::Flight fl = fx::split_flight(d.E * bg.inv_Rdt);   // eq. intinv (homogeneous)
+    st.whole_f = fl.whole;
+    st.left_f = fl.left;
+    ++st.k;
+    if (coupled) {
+        double bh2;
+        const double bh = bg.beta_hat(hs, bh2);
+        if (st.fresh) {
+            st.chi_first = d.chi;
+            st.fresh = false;
+        }
+        st.num = fma(bh, d.chi, st.num);
+        st.den += bh2;
+        const int to_end = st.Ec - st.i_f;                      // >= 0
+        if (fl.whole < to_end) {
+            const double ah = d.E + om;                           // R tau' = R tau + R zeta
+            st.num = fma(ah, d.nu, st.num);
+            st.den = fma(ah, ah, st.den);
+        } else {
+            // coarse KD step
+            const double sc = bg.Rdt * fx::steps_left(st.Ec - st.ic - st.whole_c - 1, st.left_c);
+            double Dc, hsc, omc;
+            Background<double>::kd_unit(sc, nu2, Dc, hsc, omc);
+            const double chit = st.den > 0.0 ? st.num * A::rsqrt_(st.den) : st.chi_first;
+            st.xc += fma(st.vc, st.oc, fma(Dc, chit, d.nu * omc));
+            // the coarse flight ends at the same collision, to_end steps later
+            st.oc = to_end > 0 ? fma(-fx::from_u32((uint32_t)to_end), bg.Rdt, d.E) : d.E;
+            st.whole_c = fl.whole - to_end;
+            st.left_c = fl.left;
+            if constexpr (!std::is_same<Trace, NoTrace>::value)
+                tr->coarse(d.nu, st.oc, chit);
+            st.ic = st.Ec;
+            st.vc = d.nu;
+            ++st.evc;
+            if (st.whole_c < L.n - st.ic) st.Ec = next_coarse_end(L, st.ic, st.whole_c);
+            st.num = 0.0;
+            st.den = 0.0;
+            st.fresh = true;
+        }
+    }
+    return !(fl.whole < L.n - st.i_f);
+}
+
 // One fine event; returns true when the pair has reached T.
 template <typename Real, int CPL, int RECIPE = 0, typename Trace = NoTrace>
 __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<Real> &L,
                                            const PhiloxKeys &keys, bool coupled_rt,
                                            Trace *tr = nullptr)
 {
+    if constexpr (std::is_same<Real, double>::value) {
+        return pair_event_fp64<CPL, RECIPE>(st, L, keys, coupled_rt, tr);
+    } else {
     typedef Arith<Real> A;
     const bool coupled = pair_is_coupled<Real, CPL>(coupled_rt);
     const Background<Real> &bg = L.bg;
@@ -168,13 +301,31 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
         }
     }
     return !(st.qf < (Real)(L.n - st.i_f));
+    }
 }
 
-// Alg. 1 / Alg. 2 epilogue: move both paths kinetically to T.
+// Position at T of a path without a collision before T, from the start
+// values (heterogeneous backgrounds: v0 is the velocity).
+template <typename Real, int PHYS>
+__device__ __forceinline__ Real straight_to_T(Real x0, Real v0, const LevelCtx<Real> &L)
+{
+    if constexpr (PHYS == 0 && std::is_same<Real, double>::value)
+        return position_at_T(L, x0, v0 * ((double)L.n * L.bg.Rdt));
+    else
+        return x0 + v0 * ((Real)L.n * L.bg.dt);          // pair_drift from t = 0
+}
+
+// Alg. 1 / Alg. 2 epilogue: move both paths kinetically to T, and leave
+// positions x in xf and xc.
 template <typename Real, int CPL>
 __device__ __forceinline__ void pair_drift(PairState<Real> &st, const LevelCtx<Real> &L, bool coupled_rt)
 {
     const bool coupled = pair_is_coupled<Real, CPL>(coupled_rt);
+    if constexpr (std::is_same<Real, double>::value) {
+        st.xf = position_at_T(L, st.x0, fma(st.vf, (double)max(L.n - st.i_f, 0) * L.bg.Rdt, st.xf));
+        if (coupled) st.xc = position_at_T(L, st.x0, fma(st.vc, (double)max(L.n - st.ic, 0) * L.bg.Rdt, st.xc));
+        return;
+    }
     if (st.i_f < L.n) st.xf = st.xf + st.vf * ((Real)(L.n - st.i_f) * L.bg.dt);
     if (coupled && st.ic < L.n) st.xc = st.xc + st.vc * ((Real)(L.n - st.ic) * L.bg.dt);
 }

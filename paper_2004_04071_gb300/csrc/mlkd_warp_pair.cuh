@@ -53,8 +53,10 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
     const Draw<Real> d = draw_r<Real, RECIPE>(st.k + 1u + (uint32_t)lane, st.pair_lo, st.word2,
                                               L.request, keys);
     const Real qn = d.E * bg.inv_Rdt;                          // flight after this event
-    const Real dv = bg.sigma * d.nu;                           // v_{k+1} - mu
-    const Real v1 = bg.mu + dv;
+    // FP64 state is dimensionless: v1 holds nu (see PairState)
+    constexpr bool kUnit = std::is_same<Real, double>::value;
+    const Real dv = kUnit ? d.nu : bg.sigma * d.nu;            // v_{k+1} - mu
+    const Real v1 = kUnit ? d.nu : bg.mu + dv;
     Real qp = __shfl_up_sync(kFullMask, qn, 1);                // flight before this event
     Real vp = __shfl_up_sync(kFullMask, v1, 1);
     if (lane == 0) {
@@ -89,10 +91,16 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
     const int nvalid = __popc(vmask);                          // a prefix of the lanes
     const int last = nvalid - 1;
 
-    const Real theta = bg.dt * ((Real)(sq + 1) - qp);          // eq. diffusive-time
-    Real a, dd, hs, om;
-    bg.kd_coeffs(theta, dv, a, dd, hs, om);
-    const Real dx = valid ? vp * (qp * bg.dt) + (a + dd * d.chi) : Real(0);   // eq. position-update
+    Real a, dd, hs, om, dx = Real(0);
+    if constexpr (kUnit) {
+        const double s = bg.Rdt * ((double)(sq + 1) - qp);
+        Background<double>::kd_unit(s, dv * dv, dd, hs, om);
+        if (valid) dx = fma(dd, d.chi, fma(dv, om, vp * (qp * bg.Rdt)));
+    } else {
+        const Real theta = bg.dt * ((Real)(sq + 1) - qp);      // eq. diffusive-time
+        bg.kd_coeffs(theta, dv, a, dd, hs, om);
+        dx = valid ? vp * (qp * bg.dt) + (a + dd * d.chi) : Real(0);   // eq. position-update
+    }
     st.xf = st.xf + warp_sum(dx);
 
     bool done;
@@ -158,11 +166,17 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             const Real chi_first = (p < 0 && !st.fresh) ? st.chi_first : chi_head;
             Real dxc = Real(0);
             if (trig) {
-                const Real thc = bg.dt * ((Real)(ecp - ic_pre) - qc_pre);
                 Real ac, dc, hsc, omc;
-                bg.kd_coeffs(thc, dv, ac, dc, hsc, omc);
                 const Real chit = cd > Real(0) ? cn * A::rsqrt_(cd) : chi_first;
-                dxc = vc_pre * (qc_pre * bg.dt) + (ac + dc * chit);
+                if constexpr (kUnit) {
+                    const double sc = bg.Rdt * ((double)(ecp - ic_pre) - qc_pre);
+                    Background<double>::kd_unit(sc, dv * dv, dc, hsc, omc);
+                    dxc = fma(dc, chit, fma(dv, omc, vc_pre * (qc_pre * bg.Rdt)));
+                } else {
+                    const Real thc = bg.dt * ((Real)(ecp - ic_pre) - qc_pre);
+                    bg.kd_coeffs(thc, dv, ac, dc, hsc, omc);
+                    dxc = vc_pre * (qc_pre * bg.dt) + (ac + dc * chit);
+                }
             }
             st.xc = st.xc + warp_sum(dxc);
             st.evc += (uint32_t)__popc(tmask);

@@ -50,6 +50,21 @@ extern "C" void roots(const double *x, int64_t count, double *s, double *r)
         r[i] = fx::rsqrt_normal(x[i]);
     }
 }
+extern "C" void flights(const double *q, int64_t count, int32_t *whole, uint64_t *left)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        const fx::Flight f = fx::split_flight(q[i]);
+        whole[i] = f.whole;
+        left[i] = f.left;
+    }
+}
+extern "C" void steps(const int32_t *n, const uint64_t *left, int64_t count, double *t, double *u)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        t[i] = fx::steps_left(n[i], left[i]);
+        u[i] = n[i] > 0 ? fx::from_u32((uint32_t)n[i]) : 0.0;
+    }
+}
 extern "C" void kd(const double *s, int64_t count, double *H, double *F, double *W, double *e)
 {
     for (int64_t i = 0; i < count; ++i) {
@@ -177,3 +192,30 @@ def test_coefficient_polynomials_and_exponential(fx):
     big = s >= 0.0625
     exact = np.exp(-s[big].astype(np.longdouble))
     assert np.all(np.abs(e[big] - exact) <= 0.5 * ulp(exact) + np.longdouble(2.0) ** -58)
+
+
+def test_flights_and_step_counts(fx):
+    """Whole steps and the rest of the collision's step of a flight (exact
+    down to 2^-64), and their sum back in FP64."""
+    from fractions import Fraction
+    rng = np.random.default_rng(6)
+    q = np.concatenate([[0.0, 5e-324, 2.0**-70, 2.0**-64, 2.0**-63, 0.5, np.nextafter(1.0, 0), 1.0, 1.5, 2.0, 1000.0,
+                         2.0**30 - 0.5, 2.0**31 - 1.0, 2.0**31, 2.0**52 + 1, 2.0**63, 2.0**64, 1e300],
+                        rng.uniform(0, 3, 2000), 2.0 ** rng.uniform(-60, 40, 2000)])
+    w, left = np.zeros(len(q), np.int32), np.zeros(len(q), np.uint64)
+    call(fx.flights, q, len(q), w, left)
+    for x, a, b in zip(q, w, left):
+        f = Fraction(float(x))
+        whole = f.numerator // f.denominator
+        assert a == min(whole, 2**31 - 1)
+        rest = (1 - (f - whole)) * 2**64
+        assert 0 <= rest - int(b) <= 1 or abs(rest - int(b)) < 1      # a whole step is 2^64 - 1
+    n = np.concatenate([[0, 0, 1, 2, 3, 2**30, 2**31 - 1], rng.integers(0, 2**20, 3000)]).astype(np.int32)
+    left = np.concatenate([np.array([1, 2**64 - 1, 2**64 - 1, 0, 1, 2**63, 2**64 - 1], np.uint64),
+                           rng.integers(0, 2**63, 3000).astype(np.uint64) * np.uint64(2)])
+    t, u = np.zeros(len(n)), np.zeros(len(n))
+    call(fx.steps, n, left, len(n), t, u)
+    assert np.array_equal(u, n.astype(np.float64))
+    for a, b, x in zip(n, left, t):
+        exact = Fraction(int(a)) + Fraction(int(b), 2**64)
+        assert abs(Fraction(float(x)) - exact) <= Fraction(float(np.spacing(x))) * Fraction(51, 100)
