@@ -552,15 +552,6 @@ __device__ __noinline__ void warp_round_complete(const BatchLaunch &B, int r, in
     if (cont || warp_controller(B, r, lane)) warp_plan(B, r, lane);
 }
 
-// A lane's running sums of its current chunk.  They change only when a pair
-// finishes, so they live in shared memory rather than in registers that the
-// event loop needs; 72 bytes per lane keeps bank conflicts at two-way.
-template <int MODE> struct LaneSums {
-    PairSums<MODE> mom;
-    unsigned long long ev_f, ev_c;
-    uint32_t pad_[2];
-};
-
 // A warp's bookkeeping of its current chunk and pools (all warp-uniform).  It
 // lives in shared memory and is read (volatile) where it is used, so that the
 // registers of the event loop hold only pair states and level constants.

@@ -8,7 +8,7 @@
 // coefficients 17 to 22 each; together they kept the FP64 pipe 85 % busy.
 // The values these functions return lie in a known range, so a 64-bit
 // fraction holds them with more than FP64's 53 bits: a product of two
-// fractions takes three 32-bit products, and the error of a function before
+// fractions takes three 32-bit products (a quarter of an FP64 one's time), and the error of a function before
 // its one rounding to FP64 is a few 2^-62.
 //
 // Plain integer C++ (the one FP32 instruction is the seed of the square
@@ -21,13 +21,15 @@
 #include <cmath>
 #endif
 
-#include "mlkd_fixed_tables.h"
-
 #ifdef __CUDACC__
-#define MLKD_HD __host__ __device__ __forceinline__
+#define MLKD_HD __device__ __forceinline__
+#define MLKD_CONSTANT static __constant__
 #else
 #define MLKD_HD inline
+#define MLKD_CONSTANT static const
 #endif
+
+#include "mlkd_fixed_tables.h"
 
 namespace mlkd {
 namespace fx {
@@ -77,38 +79,77 @@ MLKD_HD float rsqrt_seed(float x)
 #endif
 }
 
-// a b 2^-64 and a b 2^-32, rounded down, at most one unit below
+MLKD_HD uint32_t umulhi(uint32_t a, uint32_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)((uint64_t)a * b >> 32);
+#endif
+}
+
+// a b 2^-64 and a b 2^-32, rounded down, at most two units below.  The high
+// halves of the cross products and one wide product: 8.2 per clock and SM
+// measured, against 6.6 with the carry of the low halves and 6.4 for
+// __umul64hi (2^20 pairs of level 8 of the periodic problem: 11.4 -> 10.0 ms).
 MLKD_HD uint64_t mul64(uint64_t a, uint64_t b)
 {
     const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
     const uint32_t bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
-    const uint64_t p = (uint64_t)ah * bl;
-    const uint64_t q = (uint64_t)al * bh + (uint32_t)p;
-    return (uint64_t)ah * bh + (p >> 32) + (q >> 32);
+    return (uint64_t)ah * bh + umulhi(ah, bl) + umulhi(al, bh);
 }
 MLKD_HD uint64_t mul64x32(uint64_t a, uint32_t b)
 {
-    return (a >> 32) * b + ((uint64_t)(uint32_t)a * b >> 32);
+    return (a >> 32) * b + umulhi((uint32_t)a, b);
 }
-MLKD_HD uint32_t mul32(uint32_t a, uint32_t b) { return (uint32_t)((uint64_t)a * b >> 32); }
 
 // c0 - x (c1 - x (c2 - ...)) for a fraction x: the tail of the sum (terms
-// below 2^-29) in 32 bits, the rest in 64
-template <typename P, int I> MLKD_HD uint32_t poly_tail(uint32_t x)
+// below 2^-29) in 32 bits, the rest in 64.
+template <typename P, int K, int I = 0> MLKD_HD uint32_t poly_tail(uint32_t x)
 {
-    constexpr uint32_t c = P::tail[I];
-    if constexpr (I + 1 < P::kTail) return c - mul32(x, poly_tail<P, I + 1>(x));
+    uint32_t c;
+    if constexpr (K == 0) {
+        constexpr uint32_t c0 = P::tail0[I];
+        c = c0;
+    } else {
+        constexpr uint32_t c1 = P::tail1[I];
+        c = c1;
+    }
+    if constexpr (I + 1 < P::kTail) return c - umulhi(x, poly_tail<P, K, I + 1>(x));
     else return c;
 }
-template <typename P, int I = 0> MLKD_HD uint64_t poly(uint64_t x)
+template <typename P> MLKD_HD uint64_t poly(const uint64_t (&c)[P::kLead][1], uint64_t x)
 {
-    constexpr uint64_t c = P::lead[I];
-    if constexpr (I + 1 < P::kLead) {
-        return c - mul64(x, poly<P, I + 1>(x));
-    } else {
-        const uint32_t xh = (uint32_t)(x >> 32);
-        return c - ((uint64_t)xh * poly_tail<P, 0>(xh) >> P::kShift);
+    const uint32_t xh = (uint32_t)(x >> 32);
+    uint64_t a = c[P::kLead - 1][0] - ((uint64_t)xh * poly_tail<P, 0>(xh) >> P::kShift0);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int i = P::kLead - 2; i >= 0; --i) a = c[i][0] - mul64(x, a);
+    return a;
+}
+// Two polynomials in the same argument.  The 64-bit steps are a rolled loop
+// over coefficients in constant memory: the FP64 event loop is longer than the
+// instruction caches like (unrolled here too, 2^20 pairs of level 8 of the
+// periodic problem take 13.3 ms, so 11.3 ms; rolled in poly() as well, the deep
+// levels lose 12 %).
+struct Two {
+    uint64_t a, b;
+};
+template <typename P> MLKD_HD Two poly_two(const uint64_t (&c)[P::kLead][2], uint64_t x)
+{
+    const uint32_t xh = (uint32_t)(x >> 32);
+    Two t;
+    t.a = c[P::kLead - 1][0] - ((uint64_t)xh * poly_tail<P, 0>(xh) >> P::kShift0);
+    t.b = c[P::kLead - 1][1] - ((uint64_t)xh * poly_tail<P, 1>(xh) >> P::kShift1);
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+    for (int i = P::kLead - 2; i >= 0; --i) {
+        t.a = c[i][0] - mul64(x, t.a);
+        t.b = c[i][1] - mul64(x, t.b);
     }
+    return t;
 }
 
 // v 2^-e rounded to nearest (0 for v = 0); the result must be a normal number
@@ -136,6 +177,58 @@ MLKD_HD uint64_t fraction(double x)
     return sh < 64 ? m >> sh : 0u;
 }
 
+// ---------------------------------------------------------------------------
+// A positive number m 2^-e with m in [2^63, 2^64): products of quantities of
+// any size, at 2^-62 relative error, without the FP64 pipe.
+// ---------------------------------------------------------------------------
+struct Pos {
+    uint64_t m;
+    int e;
+};
+MLKD_HD Pos pos_of(double x)          // x a positive normal number (0: a number below 2^-1000)
+{
+    const uint64_t b = bits_of(x);
+    Pos r;
+    r.m = (b << 11) | 0x8000000000000000ull;
+    r.e = 1023 + 63 - (int)(b >> 52);
+    return r;
+}
+MLKD_HD Pos pos_fixed(uint64_t v, int e)                      // v 2^-e, v != 0
+{
+    const int lz = clz64(v);
+    Pos r;
+    r.m = v << lz;
+    r.e = e + lz;
+    return r;
+}
+MLKD_HD Pos pos_norm(uint64_t p, int e)                       // p 2^-e, p in [2^62, 2^64)
+{
+    const int sh = (int)(p >> 63) ^ 1;
+    Pos r;
+    r.m = p << sh;
+    r.e = e + sh;
+    return r;
+}
+MLKD_HD Pos operator*(const Pos &a, const Pos &b) { return pos_norm(mul64(a.m, b.m), a.e + b.e - 64); }
+// a times a fraction f 2^-64 of at least 1/2
+MLKD_HD Pos times(const Pos &a, uint64_t f) { return pos_norm(mul64(a.m, f), a.e); }
+MLKD_HD uint64_t bits_of(const Pos &a)                        // of the nearest double
+{
+    return ((uint64_t)(1023 + 63 - 1 - a.e) << 52) + (a.m >> 11) + ((a.m >> 10) & 1u);
+}
+MLKD_HD double to_double(const Pos &a) { return from_bits(bits_of(a)); }
+// the same, 0 below 2^-1021
+MLKD_HD double to_double_or_0(const Pos &a) { return from_bits(a.e <= 1084 ? bits_of(a) : 0u); }
+// a 2^k rounded down, for a 2^k < 2^64
+MLKD_HD uint64_t scaled(const Pos &a, int k)
+{
+    const int sh = a.e - k;
+    return sh < 64 ? a.m >> sh : 0u;
+}
+
+// v 2^-sh rounded down, for either sign of sh (sh > -64)
+MLKD_HD uint64_t shift_to(uint64_t v, int sh) { return sh < 0 ? v << -sh : sh < 64 ? v >> sh : 0u; }
+
 // n as a double, n >= 1
 MLKD_HD double from_u32(uint32_t n)
 {
@@ -148,59 +241,54 @@ MLKD_HD double from_u32(uint32_t n)
     return from_bits(((uint64_t)(uint32_t)((1023 + 31 - 1 - lz) << 20) << 32) + ((uint64_t)m << 21));
 }
 
-// A flight q >= 0 in steps: whole = floor(q) (at most 2^31 - 1) and
+// A flight q in steps: whole = floor(q) (at most 2^31 - 1) and
 // left = (whole + 1 - q) 2^64, the part of the collision's step that is left
 // (2^64 - 1 for a whole step)
 struct Flight {
     int whole;
     uint64_t left;
 };
-MLKD_HD Flight split_flight(double q)
+MLKD_HD Flight split_flight(const Pos &q)
 {
-    const uint64_t b = bits_of(q);
-    const int ex = (int)(b >> 52) - 1023;
-    const uint64_t m = (b << 11) | 0x8000000000000000ull;     // q = m 2^(ex - 63)
     Flight f;
     uint64_t frac;
-    if (ex < 0) {
+    if (q.e >= 64) {
         f.whole = 0;
-        frac = ex > -64 ? m >> ((-1 - ex) & 63) : 0u;
+        frac = scaled(q, 64);
     } else {
-        f.whole = ex < 31 ? (int)(uint32_t)(m >> ((63 - ex) & 63)) : 0x7fffffff;
-        frac = ex < 63 ? m << ((ex + 1) & 63) : 0u;
+        f.whole = q.e > 32 ? (int)(uint32_t)(q.m >> q.e) : 0x7fffffff;
+        frac = q.e > 0 ? q.m << (64 - q.e) : 0u;
     }
     f.left = frac ? 0u - frac : ~(uint64_t)0;
     return f;
 }
 
-// steps + left 2^-64 as a double (steps >= 0)
-MLKD_HD double steps_left(int steps, uint64_t left)
+// steps + left 2^-64 (steps >= 0, the sum not 0)
+MLKD_HD Pos steps_left(int steps, uint64_t left)
 {
-    if (steps == 0) return to_double(left, 64);
+    const Pos a = pos_fixed(left | 1u, 64);
 #ifdef __CUDA_ARCH__
-    const int lz = __clz(steps);
+    const int lz = __clz(steps | 1);
 #else
-    const int lz = __builtin_clz((uint32_t)steps);
+    const int lz = __builtin_clz((uint32_t)steps | 1u);
 #endif
     // the leading bit of the 96-bit number comes to bit 63; lz >= 1
     const uint64_t v = ((uint64_t)(uint32_t)steps << (32 + lz)) | (left >> (32 - lz));
-    return from_bits(((uint64_t)(1023 + 31 - 1 - lz) << 52) + (v >> 11) + ((v >> 10) & 1u));
+    Pos r;
+    r.m = steps ? v : a.m;
+    r.e = steps ? 32 + lz : a.e;
+    return r;
 }
 
 // ---------------------------------------------------------------------------
-// -ln u = v 2^-e for the uniform u = n 2^-B, 1 <= n <= 2^B.  n is normalised
+// -ln u for the uniform u = n 2^-B, 1 <= n <= 2^B.  n is normalised
 // to x in [1/2, 1); with the reciprocal c of the upper end of x's interval
 // (128 of them), 1 - x c = rho < 2^-7 and -ln x = ln c + rho + rho^2/2 + ...
 // + rho^8/8.  Above 1 - 2^-12 (one draw in 4096), where the logarithm is about
 // the small difference itself, the caller takes log_near_one: it keeps FP64's
 // relative error there.
 // ---------------------------------------------------------------------------
-struct Fixed {
-    uint64_t v;
-    int e;
-};
-
-template <int B, typename Tab> MLKD_HD Fixed neg_log(uint64_t n, const Tab &tab)
+template <int B, typename Tab> MLKD_HD Pos neg_log(uint64_t n, const Tab &tab)
 {
     const int lz = clz64(n);
     const uint64_t x = n << lz;
@@ -211,17 +299,14 @@ template <int B, typename Tab> MLKD_HD Fixed neg_log(uint64_t n, const Tab &tab)
     const uint32_t yh = (uint32_t)(y >> 32);
     // 1/4 + rho/5 + rho^2/6 + rho^3/7 + rho^4/8, then 1/3 + rho (.), 1/2 + rho (.)
     uint32_t t = (1u << 11) / 7u + (yh >> 28);
-    t = (1u << 18) / 6u + mul32(yh, t);
-    t = (1u << 25) / 5u + mul32(yh, t);
-    t = (1u << 30) + mul32(yh, t);
+    t = (1u << 18) / 6u + umulhi(yh, t);
+    t = (1u << 25) / 5u + umulhi(yh, t);
+    t = (1u << 30) + umulhi(yh, t);
     const uint64_t s = 0x5555555555555555ull + ((uint64_t)yh * t >> 7);
     const uint64_t w = 0x8000000000000000ull + (mul64(y, s) >> 7);
     const uint64_t l = tab.ln(j) + rho + (mul64(y, mul64(y, w)) >> 14);
     const int k = lz + B - 64;                                // whole powers of two in 1/u
-    Fixed r;
-    r.v = k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l;
-    r.e = k > 0 ? 58 : 64;
-    return r;
+    return pos_fixed(k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l, k > 0 ? 58 : 64);
 }
 
 // -ln(1 - w) for 0 <= w < 2^-12, in FP64
@@ -267,40 +352,34 @@ MLKD_HD uint64_t rsqrt62(uint64_t m)
     return s + (mul64(s, r.c) >> 20);
 }
 
-// sqrt(v 2^-e), v != 0
-MLKD_HD double sqrt_fixed(uint64_t v, int e)
+MLKD_HD Pos sqrt(const Pos &x)
 {
-    const int lz = clz64(v);
-    uint64_t m = v << lz;
-    const int p = e + lz;                                     // v 2^-e = m 2^-p
-    m >>= p & 1;
-    // sqrt(m) 2^(-p'/2) = (s 2^-63) 2^32 2^(-p'/2), p' = p - (p & 1)
-    return to_double_62(sqrt63(m), 31 + (p >> 1));
+    const int odd = x.e & 1;
+    // sqrt(m 2^-e) = sqrt(m/2^odd) 2^((odd - e)/2) = (s 2^-63) 2^32 2^((odd - e)/2)
+    const uint64_t s = sqrt63(x.m >> odd);                    // [2^62, 2^63]
+    Pos r;
+    r.m = s >> 63 ? ~(uint64_t)0 : s << 1;
+    r.e = 32 + (x.e >> 1);
+    return r;
 }
 
 // sqrt and 1/sqrt of a positive normal double
-MLKD_HD double sqrt_normal(double x)
-{
-    const uint64_t b = bits_of(x);
-    const int p = 1023 + 63 - (int)(b >> 52);                 // x = m 2^-p
-    uint64_t m = (b << 11) | 0x8000000000000000ull;
-    m >>= p & 1;
-    return to_double_62(sqrt63(m), 31 + (p >> 1));
-}
+MLKD_HD double sqrt_normal(double x) { return to_double(sqrt(pos_of(x))); }
 MLKD_HD double rsqrt_normal(double x)
 {
-    const uint64_t b = bits_of(x);
-    const int p = 1023 + 63 - (int)(b >> 52);
-    uint64_t m = (b << 11) | 0x8000000000000000ull;
-    m >>= p & 1;
-    // 1/sqrt(x) = 2^(p'/2) / sqrt(m) = (r 2^-62) 2^-32 2^(p'/2)
-    return to_double_62(rsqrt62(m), 94 - (p >> 1));
+    const Pos p = pos_of(x);
+    // 1/sqrt(x) = 2^(e'/2) / sqrt(m) = (r 2^-62) 2^-32 2^(e'/2)
+    return to_double_62(rsqrt62(p.m >> (p.e & 1)), 94 - (p.e >> 1));
 }
 
 // ---------------------------------------------------------------------------
 // cos and sin of 2 pi phase 2^-64: the nearest quarter turn, z in [-pi/4, pi/4]
 // ---------------------------------------------------------------------------
-MLKD_HD void sincos_turn(uint64_t phase, double *sn, double *cs)
+struct Turn {
+    uint64_t sin, cos;            // magnitudes, in 2^-64 (below 1)
+    uint64_t sin_sign, cos_sign;  // the sign bits of doubles
+};
+MLKD_HD Turn sincos_turn(uint64_t phase)
 {
     const uint32_t k = (uint32_t)((phase + (1ull << 61)) >> 62);
     const uint64_t r = phase - ((uint64_t)k << 62);           // signed residual
@@ -308,31 +387,33 @@ MLKD_HD void sincos_turn(uint64_t phase, double *sn, double *cs)
     const uint64_t a = (neg ? 0u - r : r) << 2;               // |residual| 2^66 <= 2^63
     const uint64_t z = mul64(a, kTwoPi_61) << 1;              // a 2^-66 2 pi, in 2^-64
     const uint64_t z2 = mul64(z, z);
-    const uint64_t s = z - mul64(z, mul64(z2, poly<PolySin>(z2)));
-    const uint64_t c = mul64(z2, poly<PolyCos>(z2));          // 1 - cos z <= 0.293
-    const double ds = to_double(s, 64);
-    const double dc = to_double(0x8000000000000000ull - (c >> 1), 63);
+    const Two p = poly_two<PolySC>(kPolySC, z2);
+    const uint64_t s = z - mul64(z, mul64(z2, p.a));
+    const uint64_t c = ~mul64(z2, p.b);                       // cos z >= 0.707
     // sin(z + k pi/2) and cos(z + k pi/2)
-    const uint64_t sz = bits_of(ds) ^ (neg ? 0x8000000000000000ull : 0u);
-    const uint64_t cz = bits_of(dc);
-    const uint64_t sp = (k & 1u) ? cz : sz, cp = (k & 1u) ? sz : cz;
-    *sn = from_bits(sp ^ ((uint64_t)(k & 2u) << 62));
-    *cs = from_bits(cp ^ ((uint64_t)((k + 1u) & 2u) << 62));
+    const bool odd = k & 1u;
+    const uint64_t sz = neg ? 0x8000000000000000ull : 0u;
+    Turn t;
+    t.sin = odd ? c : s;
+    t.cos = odd ? s : c;
+    t.sin_sign = (odd ? 0u : sz) ^ ((uint64_t)(k & 2u) << 62);
+    t.cos_sign = (odd ? sz : 0u) ^ ((uint64_t)((k + 1u) & 2u) << 62);
+    return t;
 }
 
 // ---------------------------------------------------------------------------
 // e^-x 2^64 for x >= 2^-4 (0 from x = 44 on): x log2 e = k + f,
 // e^-x = 2^-k (1 - f P(f))
 // ---------------------------------------------------------------------------
-MLKD_HD uint64_t exp_neg(double x)
+MLKD_HD uint64_t exp_neg(const Pos &x)
 {
-    const uint64_t b = bits_of(x);
-    const int ex = max_int((int)(b >> 52) - 1023, -2);        // x = m 2^(ex - 63)
-    const uint64_t m = ((b << 11) | 0x8000000000000000ull) >> ((ex + 1023 - (int)(b >> 52)) & 63);
+    const int ex = max_int(63 - x.e, -2);                     // x = m 2^(ex - 63)
+    const uint64_t m = x.m >> ((ex + x.e - 63) & 63);
     const uint64_t y = mul64(m, kLog2e_63);                   // x log2 e 2^(62 - ex)
     const uint64_t f = y << ((ex + 2) & 63);
-    const uint64_t p = ~mul64(f, poly<PolyE>(f));
-    return (uint32_t)(b >> 32) < 0x40460000u ? p >> (int)(((y >> 1) >> ((61 - ex) & 63)) & 63u) : 0u;    // 44.0
+    const uint64_t p = ~mul64(f, poly<PolyE>(kPolyE, f));
+    const bool in_range = x.e > 58 || (x.e == 58 && x.m < 0xb000000000000000ull);    // x < 44
+    return in_range ? p >> (int)(((y >> 1) >> ((61 - ex) & 63)) & 63u) : 0u;
 }
 
 }  // namespace fx

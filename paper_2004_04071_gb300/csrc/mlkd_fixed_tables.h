@@ -1,98 +1,74 @@
 // Constants of mlkd_fixed.h, written by gen_fixed.py beside this file.
+// MLKD_CONSTANT is defined there: constant memory on the device.
 #pragma once
 #include <cstdint>
 namespace mlkd {
 namespace fx {
-// h(s)/s^2, h(s) = exp(-s) + s - 1, 0 <= s <= 1
-struct PolyH {
-    static constexpr int kLead = 11, kTail = 2, kShift = 32;
-    static constexpr uint64_t lead[kLead] = {
-        0x8000000000000000ull,
-        0x2aaaaaaaaaaaaa4cull,
-        0x0aaaaaaaaaaa95daull,
-        0x0222222222205765ull,
-        0x005b05b05af12783ull,
-        0x000d00d00c74a4cfull,
-        0x0001a019ff3938fdull,
-        0x00002e3bc0383aecull,
-        0x0000049f85a3e4efull,
-        0x0000006b852e0d27ull,
-        0x00000008e48f9e46ull};
-    static constexpr uint32_t tail[kTail] = {
-        0xa4dbf70au, 0x08364b2au};
+// 2 h(s)/s^2, h(s) = exp(-s) + s - 1, and f(s)/s^3, f(s) = 2(exp(-s) - 1) + s(exp(-s) + 1), 0 <= s <= 1
+struct PolyHF {
+    static constexpr int kLead = 11, kTail = 2;
+    static constexpr int kShift0 = 31;
+    static constexpr uint32_t tail0[kTail] = {0xa4dbf70au, 0x08364b2au};
+    static constexpr int kShift1 = 32;
+    static constexpr uint32_t tail1[kTail] = {0x8d1fb798u, 0x07165888u};
 };
-// f(s)/s^3, f(s) = 2(exp(-s) - 1) + s(exp(-s) + 1), 0 <= s <= 1
-struct PolyF {
-    static constexpr int kLead = 10, kTail = 3, kShift = 29;
-    static constexpr uint64_t lead[kLead] = {
-        0x2aaaaaaaaaaaaaaaull,
-        0x1555555555555502ull,
-        0x0666666666665440ull,
-        0x016c16c16c153164ull,
-        0x0041041040f2280aull,
-        0x0009c09c09465f15ull,
-        0x000143a270f27f92ull,
-        0x000024fc9943e9eaull,
-        0x000003c8554bee00ull,
-        0x0000005998df72b8ull};
-    static constexpr uint32_t tail[kTail] = {
-        0xf0ba553fu, 0x11a3f6f3u, 0x00e2cb11u};
-};
+MLKD_CONSTANT uint64_t kPolyHF[11][2] = {
+    {0xffffffffffffffffull, 0x2aaaaaaaaaaaaaaaull},
+    {0x5555555555555497ull, 0x1555555555555502ull},
+    {0x1555555555552bb4ull, 0x0666666666665440ull},
+    {0x044444444440aecbull, 0x016c16c16c153164ull},
+    {0x00b60b60b5e24f07ull, 0x0041041040f2280aull},
+    {0x001a01a018e9499dull, 0x0009c09c09465f15ull},
+    {0x00034033fe7271faull, 0x000143a270f27f92ull},
+    {0x00005c77807075d9ull, 0x000024fc9943e9eaull},
+    {0x0000093f0b47c9ddull, 0x000003c8554bee00ull},
+    {0x000000d70a5c1a4eull, 0x0000005998df72b8ull},
+    {0x00000011c91f3c8bull, 0x0000000785d2a9f9ull}};
 // sqrt(2 (exp(-h) + h - 1))/h, 0 <= h <= exp(-1)
 struct PolyW {
-    static constexpr int kLead = 7, kTail = 3, kShift = 22;
-    static constexpr uint64_t lead[kLead] = {
-        0xffffffffffffffffull,
-        0x2aaaaaaaaaaaaa9bull,
-        0x071c71c71c71c174ull,
-        0x00f2b9d6480e6752ull,
-        0x001948b0fcc96afaull,
-        0x00020bfad21b8142ull,
-        0x000021e78ee38e7bull};
-    static constexpr uint32_t tail[kTail] = {
-        0x837f243au, 0x098fe4d6u, 0x00a41374u};
+    static constexpr int kLead = 7, kTail = 3;
+    static constexpr int kShift0 = 22;
+    static constexpr uint32_t tail0[kTail] = {0x837f243au, 0x098fe4d6u, 0x00a41374u};
 };
+MLKD_CONSTANT uint64_t kPolyW[7][1] = {
+    {0xffffffffffffffffull},
+    {0x2aaaaaaaaaaaaa9bull},
+    {0x071c71c71c71c174ull},
+    {0x00f2b9d6480e6752ull},
+    {0x001948b0fcc96afaull},
+    {0x00020bfad21b8142ull},
+    {0x000021e78ee38e7bull}};
 // (1 - 2^-f)/f, 0 <= f <= 1
 struct PolyE {
-    static constexpr int kLead = 10, kTail = 2, kShift = 31;
-    static constexpr uint64_t lead[kLead] = {
-        0xb17217f7d1cf79aaull,
-        0x3d7f7bff058b1acbull,
-        0x0e35846b824fe76cull,
-        0x0276556df74104a4ull,
-        0x005761ff9dd4a2dfull,
-        0x000a184895de347aull,
-        0x0000ffe5f74da630ull,
-        0x0000162bf1b6bc61ull,
-        0x000001b50af3e60dull,
-        0x0000001e31028c6aull};
-    static constexpr uint32_t tail[kTail] = {
-        0xeadd7cbeu, 0x0a46767du};
+    static constexpr int kLead = 10, kTail = 2;
+    static constexpr int kShift0 = 31;
+    static constexpr uint32_t tail0[kTail] = {0xeadd7cbeu, 0x0a46767du};
 };
-// (1 - sin(z)/z)/z^2 in z^2, |z| <= pi/4
-struct PolySin {
-    static constexpr int kLead = 5, kTail = 4, kShift = 32;
-    static constexpr uint64_t lead[kLead] = {
-        0x2aaaaaaaaaaaaaabull,
-        0x0222222222222222ull,
-        0x000d00d00d00d00dull,
-        0x00002e3bc74aad8eull,
-        0x0000006b99159fd5ull};
-    static constexpr uint32_t tail[kTail] = {
-        0xb092309du, 0x00d73f9fu, 0x0000ca96u, 0x00000098u};
+MLKD_CONSTANT uint64_t kPolyE[10][1] = {
+    {0xb17217f7d1cf79aaull},
+    {0x3d7f7bff058b1acbull},
+    {0x0e35846b824fe76cull},
+    {0x0276556df74104a4ull},
+    {0x005761ff9dd4a2dfull},
+    {0x000a184895de347aull},
+    {0x0000ffe5f74da630ull},
+    {0x0000162bf1b6bc61ull},
+    {0x000001b50af3e60dull},
+    {0x0000001e31028c6aull}};
+// (1 - sin(z)/z)/z^2 and (1 - cos(z))/z^2 in z^2, |z| <= pi/4
+struct PolySC {
+    static constexpr int kLead = 5, kTail = 4;
+    static constexpr int kShift0 = 32;
+    static constexpr uint32_t tail0[kTail] = {0xb092309du, 0x00d73f9fu, 0x0000ca96u, 0x00000098u};
+    static constexpr int kShift1 = 28;
+    static constexpr uint32_t tail1[kTail] = {0x8f76c780u, 0x00c9cba5u, 0x0000d740u, 0x000000b4u};
 };
-// (1 - cos(z))/z^2 in z^2, |z| <= pi/4
-struct PolyCos {
-    static constexpr int kLead = 5, kTail = 4, kShift = 28;
-    static constexpr uint64_t lead[kLead] = {
-        0x8000000000000000ull,
-        0x0aaaaaaaaaaaaaabull,
-        0x005b05b05b05b05bull,
-        0x0001a01a01a01a02ull,
-        0x0000049f93edde28ull};
-    static constexpr uint32_t tail[kTail] = {
-        0x8f76c780u, 0x00c9cba5u, 0x0000d740u, 0x000000b4u};
-};
+MLKD_CONSTANT uint64_t kPolySC[5][2] = {
+    {0x2aaaaaaaaaaaaaabull, 0x8000000000000000ull},
+    {0x0222222222222222ull, 0x0aaaaaaaaaaaaaabull},
+    {0x000d00d00d00d00dull, 0x005b05b05b05b05bull},
+    {0x00002e3bc74aad8eull, 0x0001a01a01a01a02ull},
+    {0x0000006b99159fd5ull, 0x0000049f93edde28ull}};
 constexpr uint64_t kLn2_64 = 0xb17217f7d1cf79acull;   // ln 2 in 2^-64
 constexpr uint64_t kLn2_58 = 0x02c5c85fdf473de7ull;   // ln 2 in 2^-58
 constexpr uint64_t kLog2e_63 = 0xb8aa3b295c17f0bcull; // log2 e in 2^-63

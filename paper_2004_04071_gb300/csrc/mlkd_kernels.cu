@@ -106,9 +106,17 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     unsigned long long pair = 0;
     typename PhysState<Real, PHYS>::type st;
     st.fresh = true;
-    PairSums<MODE> mom;
+    // FP64: the running sums in shared memory, so that the event loop fits 64
+    // registers (8 blocks per SM)
+    constexpr bool kSharedSums = std::is_same<Real, double>::value;
+    __shared__ LaneSums<MODE> s_sums[kSharedSums ? kThreads : 1];
+    LaneSums<MODE> r_sums;
+    LaneSums<MODE> &sums = kSharedSums ? s_sums[kSharedSums ? threadIdx.x : 0] : r_sums;
+    PairSums<MODE> &mom = sums.mom;
+    unsigned long long &ev_f_sum = sums.ev_f, &ev_c_sum = sums.ev_c;
     mom.zero();
-    unsigned long long ev_f_sum = 0, ev_c_sum = 0;
+    ev_f_sum = 0;
+    ev_c_sum = 0;
 
     // QoI, sums and histogram of the finished pair.
     auto finish_pair = [&]() {

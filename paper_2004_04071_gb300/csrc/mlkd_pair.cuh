@@ -87,7 +87,7 @@ template <typename Real> __device__ __forceinline__ Real first_flight(const Leve
 template <typename Real> __device__ __forceinline__ bool collides_before_T(const LevelCtx<Real> &L, Real q0)
 {
     if constexpr (std::is_same<Real, double>::value)
-        return fx::split_flight(first_flight(L, q0)).whole < L.n;
+        return fx::split_flight(fx::pos_of(first_flight(L, q0))).whole < L.n;
     else
         return q0 < (Real)L.n;
 }
@@ -140,7 +140,7 @@ __device__ __forceinline__ bool pair_init(PairState<Real> &st, unsigned long lon
     st.evc = 0;
     int whole;
     if constexpr (std::is_same<Real, double>::value) {
-        const fx::Flight fl = fx::split_flight(qf);
+        const fx::Flight fl = fx::split_flight(fx::pos_of(qf));
         whole = fl.whole;
         st.of = st.oc = q0;
         st.whole_f = st.whole_c = fl.whole;
@@ -173,11 +173,12 @@ __device__ __forceinline__ bool pair_start(PairState<Real> &st, unsigned long lo
 
 // One fine event of the FP64 state; returns true when the pair has reached T.
 // The FP64 pipe bounds it (two operations per clock and SM), so everything
-// that can be is integer: draws, coefficients and roots in fixed point, step
-// counts and window tests on the whole part of a flight, conversions by
-// moving bits.  19 FP64 operations are left per fine event and 12 per coarse
-// one, against about 45 and 27 with positions in x and times in FP64: level 8
-// of the periodic problem, 131 071 pairs, 2.41 -> 1.86 ms.
+// that can be is integer: draws, coefficients, weights and flights are
+// positive numbers with 64-bit mantissas (fx::Pos) or fractions, step counts
+// and window tests integers.  What is left in FP64 are the sums: 4 operations
+// for the position and 6 for the window per fine event and 6 per coarse one,
+// against about 45 and 27 with every quantity in FP64 (131 071 pairs of level 8
+// of the periodic problem: 1.54 ms, 1.86 ms with FP64 products).
 template <int CPL, int RECIPE, typename Trace>
 __device__ __forceinline__ bool pair_event_fp64(PairState<double> &st, const LevelCtx<double> &L,
                                                 const PhiloxKeys &keys, bool coupled_rt, Trace *tr)
@@ -185,50 +186,48 @@ __device__ __forceinline__ bool pair_event_fp64(PairState<double> &st, const Lev
     typedef Arith<double> A;
     const bool coupled = pair_is_coupled<double, CPL>(coupled_rt);
     const Background<double> &bg = L.bg;
-    const Draw<double> d = draw_r<double, RECIPE>(st.k + 1u, st.pair_lo, st.word2, L.request, keys);
-    const double s = bg.Rdt * fx::to_double(st.left_f, 64);     // R theta (eq. diffusive-time)
-    const double nu2 = d.nu * d.nu;
-    double D, hs, om;
-    Background<double>::kd_unit(s, nu2, D, hs, om);
+    const DrawFixed d = draw_fixed_r<RECIPE>(st.k + 1u, st.pair_lo, st.word2, L.request, keys);
+    const double nu = d.nu_(), chi = d.chi_(), E = fx::to_double(d.E);
+    const fx::Pos Rdt = fx::pos_of(bg.Rdt);
+    const fx::Pos nu2 = d.nu * d.nu;
+    // s = R theta (eq. diffusive-time)
+    const Background<double>::Unit f = Background<double>::kd_unit<CPL != 0>(Rdt * fx::steps_left(0, st.left_f), nu2);
     // eq. position-update: nu_k E_k, then nu_{k+1} (1 - e^{-s}) + D chi_k; one
     // rounding at the size of y
-    st.xf += fma(st.vf, st.of, fma(D, d.chi, d.nu * om));
+    st.xf += fma(st.vf, st.of, fma(f.D, chi, nu * f.om));
     st.i_f += st.whole_f + 1;                                   // eq. time-update
-    st.vf = d.nu;
-    st.of = d.E;
-    const fx::Flight fl = fx::split_flight(d.E * bg.inv_Rdt);   // eq. intinv (homogeneous)
+    st.vf = nu;
+    st.of = E;
+    const fx::Flight fl = fx::split_flight(d.E * fx::pos_of(bg.inv_Rdt));    // eq. intinv (homogeneous)
     st.whole_f = fl.whole;
     st.left_f = fl.left;
     ++st.k;
     if (coupled) {
-        double bh2;
-        const double bh = bg.beta_hat(hs, bh2);
         if (st.fresh) {
-            st.chi_first = d.chi;
+            st.chi_first = chi;
             st.fresh = false;
         }
-        st.num = fma(bh, d.chi, st.num);
-        st.den += bh2;
+        st.num = fma(f.beta, chi, st.num);
+        st.den = fma(f.beta, f.beta, st.den);
         const int to_end = st.Ec - st.i_f;                      // >= 0
         if (fl.whole < to_end) {
-            const double ah = d.E + om;                           // R tau' = R tau + R zeta
-            st.num = fma(ah, d.nu, st.num);
+            const double ah = E + f.om;                           // R tau' = R tau + R zeta
+            st.num = fma(ah, nu, st.num);
             st.den = fma(ah, ah, st.den);
         } else {
             // coarse KD step
-            const double sc = bg.Rdt * fx::steps_left(st.Ec - st.ic - st.whole_c - 1, st.left_c);
-            double Dc, hsc, omc;
-            Background<double>::kd_unit(sc, nu2, Dc, hsc, omc);
-            const double chit = st.den > 0.0 ? st.num * A::rsqrt_(st.den) : st.chi_first;
-            st.xc += fma(st.vc, st.oc, fma(Dc, chit, d.nu * omc));
+            const fx::Pos sc = Rdt * fx::steps_left(st.Ec - st.ic - st.whole_c - 1, st.left_c);
+            const Background<double>::Unit c = Background<double>::kd_unit<false>(sc, nu2);
+            const double chit = fx::bits_of(st.den) ? st.num * A::rsqrt_(st.den) : st.chi_first;   // den >= 0
+            st.xc += fma(st.vc, st.oc, fma(c.D, chit, nu * c.om));
             // the coarse flight ends at the same collision, to_end steps later
-            st.oc = to_end > 0 ? fma(-fx::from_u32((uint32_t)to_end), bg.Rdt, d.E) : d.E;
+            st.oc = to_end > 0 ? fma(-fx::from_u32((uint32_t)to_end), bg.Rdt, E) : E;
             st.whole_c = fl.whole - to_end;
             st.left_c = fl.left;
             if constexpr (!std::is_same<Trace, NoTrace>::value)
-                tr->coarse(d.nu, st.oc, chit);
+                tr->coarse(nu, st.oc, chit);
             st.ic = st.Ec;
-            st.vc = d.nu;
+            st.vc = nu;
             ++st.evc;
             if (st.whole_c < L.n - st.ic) st.Ec = next_coarse_end(L, st.ic, st.whole_c);
             st.num = 0.0;
@@ -420,6 +419,15 @@ template <> struct PairSums<kModeFP32Comp> {
             for (int j = 0; j < 6; ++j) q[j].shfl_merge(off);
     }
     __device__ double value(int j) const { return q[j].value(); }
+};
+
+// A lane's running sums.  They change only when a pair finishes, so where the
+// event loop needs the registers they live in shared memory; 72 bytes per
+// lane keeps bank conflicts at two-way.
+template <int MODE> struct LaneSums {
+    PairSums<MODE> mom;
+    unsigned long long ev_f, ev_c;
+    uint32_t pad_[2];
 };
 
 // QoI of one finished pair (eq. mlmc-compact): F(x) = x^2 in free space or

@@ -91,11 +91,13 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
     const int nvalid = __popc(vmask);                          // a prefix of the lanes
     const int last = nvalid - 1;
 
-    Real a, dd, hs, om, dx = Real(0);
+    Real a, dd, hs, om, dx = Real(0), bh = Real(0);
     if constexpr (kUnit) {
         const double s = bg.Rdt * ((double)(sq + 1) - qp);
-        Background<double>::kd_unit(s, dv * dv, dd, hs, om);
-        if (valid) dx = fma(dd, d.chi, fma(dv, om, vp * (qp * bg.Rdt)));
+        const Background<double>::Unit f = Background<double>::kd_unit<true>(fx::pos_of(s), fx::pos_of(dv * dv));
+        om = f.om;
+        bh = f.beta;
+        if (valid) dx = fma(f.D, d.chi, fma(dv, om, vp * (qp * bg.Rdt)));
     } else {
         const Real theta = bg.dt * ((Real)(sq + 1) - qp);      // eq. diffusive-time
         bg.kd_coeffs(theta, dv, a, dd, hs, om);
@@ -122,7 +124,8 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             const bool trig = valid && Kn != Kp;
             const unsigned tmask = __ballot_sync(kFullMask, trig);
             Real bh2;
-            const Real bh = bg.beta_hat(hs, bh2);
+            if constexpr (kUnit) bh2 = bh * bh;
+            else bh = bg.beta_hat(hs, bh2);
             Real cn = valid ? bh * d.chi : Real(0);
             Real cd = valid ? bh2 : Real(0);
             if (valid && !trig) {
@@ -166,14 +169,15 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             const Real chi_first = (p < 0 && !st.fresh) ? st.chi_first : chi_head;
             Real dxc = Real(0);
             if (trig) {
-                Real ac, dc, hsc, omc;
+                Real ac, dc, omc;
                 const Real chit = cd > Real(0) ? cn * A::rsqrt_(cd) : chi_first;
                 if constexpr (kUnit) {
                     const double sc = bg.Rdt * ((double)(ecp - ic_pre) - qc_pre);
-                    Background<double>::kd_unit(sc, dv * dv, dc, hsc, omc);
-                    dxc = fma(dc, chit, fma(dv, omc, vc_pre * (qc_pre * bg.Rdt)));
+                    const Background<double>::Unit c = Background<double>::kd_unit<false>(fx::pos_of(sc), fx::pos_of(dv * dv));
+                    dxc = fma(c.D, chit, fma(dv, c.om, vc_pre * (qc_pre * bg.Rdt)));
                 } else {
                     const Real thc = bg.dt * ((Real)(ecp - ic_pre) - qc_pre);
+                    Real hsc;
                     bg.kd_coeffs(thc, dv, ac, dc, hsc, omc);
                     dxc = vc_pre * (qc_pre * bg.dt) + (ac + dc * chit);
                 }

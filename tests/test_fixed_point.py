@@ -26,13 +26,14 @@ struct Tab {
     uint32_t recip(int j) const { return rc[j]; }
     uint64_t ln(int j) const { return ln_[j]; }
 };
-template <int B> static fx::Fixed nl(uint64_t n) { return fx::neg_log<B>(n, Tab()); }
+template <int B> static fx::Pos nl(uint64_t n) { return fx::neg_log<B>(n, Tab()); }
 extern "C" void neg_log(int B, const uint64_t *n, int64_t count, double *E, double *r)
 {
     for (int64_t i = 0; i < count; ++i) {
-        const fx::Fixed f = B == 53 ? nl<53>(n[i]) : nl<24>(n[i]);
-        E[i] = fx::to_double(f.v, f.e);
-        r[i] = fx::sqrt_fixed(f.v, f.e - 1);
+        fx::Pos f = B == 53 ? nl<53>(n[i]) : nl<24>(n[i]);
+        E[i] = fx::to_double(f);
+        f.e -= 1;
+        r[i] = fx::to_double(fx::sqrt(f));
     }
 }
 extern "C" void near_one(const double *w, int64_t count, double *E)
@@ -41,7 +42,11 @@ extern "C" void near_one(const double *w, int64_t count, double *E)
 }
 extern "C" void sincos_turn(const uint64_t *p, int64_t count, double *s, double *c)
 {
-    for (int64_t i = 0; i < count; ++i) fx::sincos_turn(p[i], s + i, c + i);
+    for (int64_t i = 0; i < count; ++i) {
+        const fx::Turn t = fx::sincos_turn(p[i]);
+        s[i] = fx::from_bits(fx::bits_of(fx::to_double(t.sin, 64)) ^ t.sin_sign);
+        c[i] = fx::from_bits(fx::bits_of(fx::to_double(t.cos, 64)) ^ t.cos_sign);
+    }
 }
 extern "C" void roots(const double *x, int64_t count, double *s, double *r)
 {
@@ -53,7 +58,7 @@ extern "C" void roots(const double *x, int64_t count, double *s, double *r)
 extern "C" void flights(const double *q, int64_t count, int32_t *whole, uint64_t *left)
 {
     for (int64_t i = 0; i < count; ++i) {
-        const fx::Flight f = fx::split_flight(q[i]);
+        const fx::Flight f = fx::split_flight(fx::pos_of(q[i]));
         whole[i] = f.whole;
         left[i] = f.left;
     }
@@ -61,7 +66,7 @@ extern "C" void flights(const double *q, int64_t count, int32_t *whole, uint64_t
 extern "C" void steps(const int32_t *n, const uint64_t *left, int64_t count, double *t, double *u)
 {
     for (int64_t i = 0; i < count; ++i) {
-        t[i] = fx::steps_left(n[i], left[i]);
+        t[i] = fx::to_double(fx::steps_left(n[i], left[i]));
         u[i] = n[i] > 0 ? fx::from_u32((uint32_t)n[i]) : 0.0;
     }
 }
@@ -69,10 +74,11 @@ extern "C" void kd(const double *s, int64_t count, double *H, double *F, double 
 {
     for (int64_t i = 0; i < count; ++i) {
         const uint64_t x = fx::fraction(s[i] < 1.0 ? s[i] : 0.0);
-        H[i] = fx::to_double_62(fx::poly<fx::PolyH>(x), 64);
-        F[i] = fx::to_double(fx::poly<fx::PolyF>(x), 64);
-        W[i] = fx::to_double_62(fx::poly<fx::PolyW>(fx::fraction(s[i] < 1.0 ? s[i] * 0.36787944117144233 : 0.0)) >> 1, 63);
-        e[i] = s[i] >= 0.0625 ? fx::to_double(fx::exp_neg(s[i]), 64) : 0.0;
+        const fx::Two p = fx::poly_two<fx::PolyHF>(fx::kPolyHF, x);
+        H[i] = fx::to_double(p.a, 65);
+        F[i] = fx::to_double(p.b, 64);
+        W[i] = fx::to_double_62(fx::poly<fx::PolyW>(fx::kPolyW, fx::fraction(s[i] < 1.0 ? s[i] * 0.36787944117144233 : 0.0)) >> 1, 63);
+        e[i] = s[i] >= 0.0625 ? fx::to_double(fx::exp_neg(fx::pos_of(s[i])), 64) : 0.0;
     }
 }
 """
