@@ -30,7 +30,10 @@ struct NoTrace {};
 // xf, xc hold y and vf, vc hold nu.  One pair per lane keeps a flight as its
 // optical length and its split into whole steps and the rest of the
 // collision's step; one pair per warp keeps it as qf, qc.
-template <typename Real> struct FlightState {};
+// FP32 keeps its floor beside qf.
+template <typename Real> struct FlightState {
+    int whole_f;                // floor(qf)
+};
 template <> struct FlightState<double> {
     double x0;                  // initial position
     double of, oc;              // optical lengths E of the fine and coarse flights
@@ -146,7 +149,7 @@ __device__ __forceinline__ bool pair_init(PairState<Real> &st, unsigned long lon
         st.whole_f = st.whole_c = fl.whole;
         st.left_f = st.left_c = fl.left;
     } else {
-        whole = (int)qf;
+        whole = st.whole_f = __float2int_rz(qf);
     }
     if (coupled) {
         st.vc = v0;
@@ -251,7 +254,7 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
     const bool coupled = pair_is_coupled<Real, CPL>(coupled_rt);
     const Background<Real> &bg = L.bg;
     const Draw<Real> d = draw_r<Real, RECIPE>(st.k + 1u, st.pair_lo, st.word2, L.request, keys);
-    const int sq = (int)st.qf;                                  // floor: qf >= 0
+    const int sq = st.whole_f;                                  // floor: qf >= 0
     const Real theta = bg.dt * ((Real)(sq + 1) - st.qf);        // eq. diffusive-time
     const Real dv = bg.sigma * d.nu;                            // v_{k+1} - mu
     const Real v1 = bg.mu + dv;
@@ -261,6 +264,11 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
     st.i_f += sq + 1;                                           // eq. time-update
     st.vf = v1;
     st.qf = d.E * bg.inv_Rdt;                                   // eq. intinv (homogeneous)
+    // The window and horizon tests compare whole steps: qf < K for an integer
+    // K exactly when floor(qf) < K.  (Conversions of step counts run at a
+    // quarter of the issue rate; the flight past T saturates.)
+    const int whole = __float2int_rz(st.qf);
+    st.whole_f = whole;
     ++st.k;
 
     if (coupled) {
@@ -274,7 +282,8 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
         }
         st.num += bh * d.chi;
         st.den += bh2;
-        if (st.qf < (Real)(st.Ec - st.i_f)) {
+        const int to_end = st.Ec - st.i_f;
+        if (whole < to_end) {
             const Real ah = st.qf * bg.Rdt + om;                  // R tau' = R tau + R zeta
             st.num += ah * d.nu;
             st.den += ah * ah;
@@ -287,19 +296,19 @@ __device__ __forceinline__ bool pair_event(PairState<Real> &st, const LevelCtx<R
             bg.kd_coeffs(thc, dv, ac, dc, hsc, omc);
             const Real chit = st.den > Real(0) ? st.num * A::rsqrt_(st.den) : st.chi_first;
             st.xc = st.xc + st.vc * (st.qc * bg.dt) + (ac + dc * chit);
-            st.qc = st.qf - (Real)(st.Ec - st.i_f);
+            st.qc = st.qf - (Real)to_end;                         // exact before T
             if constexpr (!std::is_same<Trace, NoTrace>::value)
                 tr->coarse(d.nu, st.qc * bg.Rdt, chit);      // nu~, E~ = R tau~, chi~
             st.ic = st.Ec;
             st.vc = v1;
             ++st.evc;
-            if (st.qc < (Real)(L.n - st.ic)) st.Ec = next_coarse_end(L, st.ic, (int)st.qc);
+            if (whole - to_end < L.n - st.ic) st.Ec = next_coarse_end(L, st.ic, whole - to_end);
             st.num = Real(0);
             st.den = Real(0);
             st.fresh = true;
         }
     }
-    return !(st.qf < (Real)(L.n - st.i_f));
+    return !(whole < L.n - st.i_f);
     }
 }
 
