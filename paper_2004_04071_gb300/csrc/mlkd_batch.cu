@@ -39,7 +39,9 @@ namespace mlkd {
 constexpr int kBL = MLKD_MAX_LEVELS;            // levels per request
 constexpr int kMaxChunksPerJob = 2048;           // chunks per level and round, at most
 constexpr int kChunkQuantum = 32;                // chunk sizes are multiples of one pair per lane
-constexpr int kTargetIters = 1024;               // target warp iterations per chunk
+constexpr int kTargetIters = 1024;               // target warp iterations per chunk of a large round
+constexpr int kMinTargetIters = 16;              // and of the smallest round
+constexpr double kRoundSpread = 8192.0;          // chunks a round of less work is spread over
 constexpr double kPairStartIters = 2.0;          // start + summation of a pair, in event iterations
 constexpr long long kMaxChunkPairs = 1LL << 22;  // pairs per chunk at most
 constexpr long long kMaxChunkGrow = 8;           // chunk enlargement to fit a round, at most
@@ -251,14 +253,26 @@ __device__ __forceinline__ unsigned long long vload64(const unsigned long long *
     return *(volatile const unsigned long long *)p;
 }
 
+// Warp iterations per chunk of a round with this much work (pairs times events
+// per pair, starts included).  A small round is split finer, so that it keeps
+// every warp of the GPU busy and ends after about one chain instead of one
+// warp's kTargetIters iterations (8 small FP64 requests in one call: 14.6 ms with
+// kTargetIters for every round, 4.8 ms; 4096 or 16384 chunks and 64 iterations
+// at least are within 2 %, or slower).  It depends on the request's own round
+// only.
+__device__ double round_target_iters(double work)
+{
+    return fmin(fmax(work / (32.0 * kRoundSpread), (double)kMinTargetIters), (double)kTargetIters);
+}
+
 // Target chunk size of a level: a multiple of 32 pairs sized for about
-// kTargetIters warp iterations.
-__device__ long long chunk_target(double events_per_pair)
+// `iters` warp iterations.
+__device__ long long chunk_target(double events_per_pair, double iters)
 {
     // a pair costs its events plus its start (draw, initial position) and
     // its summation, about two event iterations together
     const double per_pair = (events_per_pair > 1.0 ? events_per_pair : 1.0) + kPairStartIters;
-    double ch = 32.0 * kTargetIters / per_pair;
+    double ch = 32.0 * iters / per_pair;
     long long c = (long long)ch / kChunkQuantum * kChunkQuantum;
     if (c < kChunkQuantum) c = kChunkQuantum;
     if (c > kMaxChunkPairs) c = kMaxChunkPairs;
@@ -436,6 +450,7 @@ __device__ __noinline__ void warp_plan(const BatchLaunch &B, int r, int lane)
     if (lane == 0) {
         long long *want = S.plan_want, *tch = S.job_ch;
         double *epps = S.plan_epp;
+        double planned = 0.0;
         for (int l = 0; l < nl; ++l) {
             want[l] = S.target[l] - S.have[l];
             if (want[l] < 0) want[l] = 0;
@@ -448,8 +463,10 @@ __device__ __noinline__ void warp_plan(const BatchLaunch &B, int r, int lane)
                 epp = (coll < nf ? coll : nf) * (l > 0 ? 1.5 : 1.0);
             }
             epps[l] = epp;
-            tch[l] = chunk_target(epp);
+            planned += (double)want[l] * (epp + kPairStartIters);
         }
+        const double iters = round_target_iters(planned);
+        for (int l = 0; l < nl; ++l) tch[l] = chunk_target(epps[l], iters);
         int total = 0;
         double work = 0.0;
         for (int l = nl - 1; l >= 0; --l) {
@@ -458,13 +475,13 @@ __device__ __noinline__ void warp_plan(const BatchLaunch &B, int r, int lane)
             long long count = want[l];
             if (count <= 0) continue;
             // A level whose pairs are long serial chains runs one pair per
-            // warp, 32 events per step; its chunks then hold about
-            // kTargetIters warp steps of pairs, not a multiple of 32.  (The
+            // warp, 32 events per step; its chunks then hold about `iters`
+            // warp steps of pairs, not a multiple of 32.  (The
             // heterogeneous backgrounds always run one pair per lane.)
             const bool wp = B.warp_pair_events > 0 && epps[l] >= (double)B.warp_pair_events &&
                             D.background == 0;
             if (wp) {
-                double c = 32.0 * kTargetIters / (epps[l] + 32.0 * kPairStartIters);
+                double c = 32.0 * iters / (epps[l] + 32.0 * kPairStartIters);
                 tch[l] = c < 1.0 ? 1 : (long long)c;
             }
             S.job_warp[l] = wp ? 1 : 0;
