@@ -85,6 +85,7 @@ def main():
     print("constexpr uint64_t kLn2_58 = 0x%016xull;   // ln 2 in 2^-58" % int(mp.nint(mp.log(2) * mp.mpf(2) ** 58)))
     print("constexpr uint64_t kLog2e_63 = 0x%016xull; // log2 e in 2^-63" % int(mp.nint(mp.mpf(2) ** 63 / mp.log(2))))
     print("constexpr uint64_t kTwoPi_61 = 0x%016xull; // 2 pi in 2^-61" % int(mp.nint(2 * mp.pi * mp.mpf(2) ** 61)))
+    print("constexpr uint64_t kInvTwoPi_64 = 0x%016xull; // 1/(2 pi) in 2^-64" % int(mp.nint(TWO64 / (2 * mp.pi))))
     # log: reciprocals of the upper ends of 128 intervals of [1/2, 1), and their logarithms
     C = [(1 << 23) // (129 + j) for j in range(128)]
     print("// floor(2^15 256/(129 + j)) and ln of that fraction, in 2^-64")

@@ -576,7 +576,7 @@ struct WarpCtx {
     unsigned long long c;            // chunk id
     unsigned long long first, end;   // the chunk's pair range
     unsigned long long next;         // next pair of the chunk to start
-    double blo, bhi, bh;             // histogram range and bin width (FP64 state)
+    double blo, bhi, bh, binv_h;     // histogram range, bin width and its inverse (FP64 state)
     float blo_f, bhi_f, binv_h_f;    // the same for FP32 state
     int32_t req, level, warp_pair, nbins, per, fkind;
     int32_t sp_n, sp_i, fp_n;        // start pool: started, handed out; finish pool: queued
@@ -690,6 +690,7 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
             X.blo = D->bd[level].lo;
             X.bhi = D->bd[level].hi;
             X.bh = D->h;
+            X.binv_h = D->bd[level].inv_h;
             X.blo_f = D->bf[level].lo;
             X.bhi_f = D->bf[level].hi;
             X.binv_h_f = D->bf[level].inv_h;
@@ -720,6 +721,7 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
             bins.lo = X.blo;
             bins.hi = X.bhi;
             bins.h = X.bh;
+            bins.inv_h = X.binv_h;
             bins.lo_f = X.blo_f;
             bins.hi_f = X.bhi_f;
             bins.inv_h_f = X.binv_h_f;

@@ -73,6 +73,7 @@ constexpr uint64_t kLn2_64 = 0xb17217f7d1cf79acull;   // ln 2 in 2^-64
 constexpr uint64_t kLn2_58 = 0x02c5c85fdf473de7ull;   // ln 2 in 2^-58
 constexpr uint64_t kLog2e_63 = 0xb8aa3b295c17f0bcull; // log2 e in 2^-63
 constexpr uint64_t kTwoPi_61 = 0xc90fdaa22168c235ull; // 2 pi in 2^-61
+constexpr uint64_t kInvTwoPi_64 = 0x28be60db9391054aull; // 1/(2 pi) in 2^-64
 // floor(2^15 256/(129 + j)) and ln of that fraction, in 2^-64
 #define MLKD_LOG_RECIPROCALS \
     65027u, 64527u, 64035u, 63550u, 63072u, 62601u, 62137u, 61680u, 61230u, 60787u, 60349u, 59918u, \

@@ -85,6 +85,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     bins.lo = P.lo;
     bins.hi = P.hi;
     bins.h = P.h;
+    bins.inv_h = P.bd.inv_h;
     bins.lo_f = P.bf.lo;
     bins.hi_f = P.bf.hi;
     bins.inv_h_f = P.bf.inv_h;

@@ -102,13 +102,15 @@ template <typename Real, int RECIPE = 0>
 __device__ __forceinline__ void pair_start_values(Real &x0, Real &v0, Real &q0, unsigned long long p,
                                                   const LevelCtx<Real> &L, const PhiloxKeys &keys)
 {
-    const Draw<Real> d0 = draw_r<Real, RECIPE>(0u, (uint32_t)p, L.word2 ^ (uint32_t)(p >> 32),
-                                               L.request, keys);
-    x0 = L.init ? cosine_inverse<Real>(d0.u4) : Real(0);
     if constexpr (std::is_same<Real, double>::value) {
-        v0 = d0.nu;
-        q0 = d0.E;
+        const DrawFixed d0 = draw_fixed_r<RECIPE>(0u, (uint32_t)p, L.word2 ^ (uint32_t)(p >> 32), L.request, keys);
+        x0 = L.init ? cosine_inverse_fp64<RECIPE == 1 ? 24 : 53>(d0.n4) : 0.0;
+        v0 = d0.nu_();
+        q0 = fx::to_double(d0.E);
     } else {
+        const Draw<Real> d0 = draw_r<Real, RECIPE>(0u, (uint32_t)p, L.word2 ^ (uint32_t)(p >> 32),
+                                                   L.request, keys);
+        x0 = L.init ? cosine_inverse<Real>(d0.u4) : Real(0);
         v0 = L.bg.mu + L.bg.sigma * d0.nu;
         q0 = d0.E * L.bg.inv_Rdt;
     }
@@ -453,8 +455,10 @@ __device__ __forceinline__ void add_pair(PairSums<kModeFP64> &ps, double xf, dou
     ps.v[1] += y * y;
     ps.v[2] += Ff;
     ps.v[3] += Ff * Ff;
-    ps.v[4] += Fc;
-    ps.v[5] += Fc * Fc;
+    if (coupled) {
+        ps.v[4] += Fc;
+        ps.v[5] += Fc * Fc;
+    }
 }
 
 __device__ __forceinline__ void add_pair(PairSums<kModeFP32DY64> &ps, float xf, float xc, bool coupled,
@@ -469,8 +473,10 @@ __device__ __forceinline__ void add_pair(PairSums<kModeFP32DY64> &ps, float xf, 
     const float Ff = mf * mf, Fc = coupled ? mc * mc : 0.0f;
     ps.q[0].add(Ff);
     ps.q[1].add(Ff * Ff);
-    ps.q[2].add(Fc);
-    ps.q[3].add(Fc * Fc);
+    if (coupled) {
+        ps.q[2].add(Fc);
+        ps.q[3].add(Fc * Fc);
+    }
 }
 
 __device__ __forceinline__ void add_pair(PairSums<kModeFP32Comp> &ps, float xf, float xc, bool coupled,
@@ -484,8 +490,10 @@ __device__ __forceinline__ void add_pair(PairSums<kModeFP32Comp> &ps, float xf, 
     ps.q[1].add(y * y);
     ps.q[2].add(Ff);
     ps.q[3].add(Ff * Ff);
-    ps.q[4].add(Fc);
-    ps.q[5].add(Fc * Fc);
+    if (coupled) {
+        ps.q[4].add(Fc);
+        ps.q[5].add(Fc * Fc);
+    }
 }
 
 // Linear QoI F(x) = x (the position at T, the paper's test case): Y = x_f -
@@ -539,14 +547,20 @@ __device__ __forceinline__ void add_pair_fk(Sums &ps, Real xf, Real xc, bool cou
 // positions are first wrapped into [0, 1).  FP64 state divides in FP64; FP32
 // state decides its bins in FP32.
 struct Bins {
-    double lo, hi, h;
+    double lo, hi, h, inv_h;
     float lo_f, hi_f, inv_h_f;
     int nbins;
     bool periodic;
     __device__ int operator()(double x) const {
         if (periodic) x = x - floor(x);
         if (!(x >= lo && x < hi)) return -1;
-        const int b = (int)floor((x - lo) / h);
+        // (x - lo)/h decided by the product with 1/h unless that comes within
+        // 2^-40 of an integer (an FP64 quotient costs ten products)
+        const double q = (x - lo) * inv_h;
+        const double t = __dadd_rd(q, 4503599627370496.0);               // 2^52 + floor(q)
+        int b = __double2loint(t);
+        const double f = q - (t - 4503599627370496.0);
+        if (!(f > 0x1p-40 && f < 1.0 - 0x1p-40)) b = (int)floor((x - lo) / h);
         return b < nbins ? b : nbins - 1;
     }
     __device__ int operator()(float x) const {
