@@ -225,7 +225,11 @@ template <typename Real, int MODE, int PPT, int PHYS = 0> constexpr int lane_wor
 // scheduler with fewer warps finishes its chain sooner; measured on the
 // periodic benchmark, five balances that against latency hiding best.
 template <typename Real, int PPT> struct BatchMinBlocks { static constexpr int value = PPT == 1 ? 5 : PPT == 2 ? 4 : PPT == 4 ? 2 : 1; };
-template <int PPT> struct BatchMinBlocks<double, PPT> { static constexpr int value = 1; };
+// FP64: four blocks (128 registers); with one (255 registers, two resident) the
+// integer arithmetic of the events hides less latency: an adaptive FP64
+// estimate of the periodic problem (eps = 0.1, tol 4e-3) takes 6.4 ms, 8.0 with
+// one, 6.6 with three, 6.8 with five.
+template <int PPT> struct BatchMinBlocks<double, PPT> { static constexpr int value = 4; };
 
 template <typename Real> __device__ __forceinline__ const BgParams<Real> &req_params(const ReqDesc &D, int l);
 template <> __device__ __forceinline__ const BgParams<float> &req_params<float>(const ReqDesc &D, int l) { return D.bf[l]; }
