@@ -507,8 +507,8 @@ MLKD_API mlkd_status mlkd_server_stop(mlkd_context *ctx);
  * and synchronisation are as for mlkd_run_level; the call uses the current
  * CUDA device and calls no device allocator.  Event counts and histogram
  * counts equal mlkd_run_level's exactly.  The floating-point sums equal them
- * bit for bit while the grid of mlkd_run_level (SMs x resident blocks, at
- * most 4096) fits under MLKD_NOALLOC_MAX_BLOCKS; where the cap binds, the
+ * bit for bit while the grid of mlkd_run_level (at most two times SMs x
+ * resident blocks, and 4096) fits under MLKD_NOALLOC_MAX_BLOCKS; where the cap binds, the
  * pairs are split over fewer blocks and the sums agree to rounding only. */
 #define MLKD_NOALLOC_MAX_BLOCKS 2048
 #define MLKD_NOALLOC_MAX_BINS 256

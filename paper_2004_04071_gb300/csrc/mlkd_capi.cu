@@ -232,19 +232,37 @@ void fill_launch(const mlkd_problem *p, const Derived &d, int j, uint64_t first,
 
 namespace {
 
-// Grid of the pair kernel: enough warps for the pairs, at most one full wave
-// of resident blocks; each warp gets an equal contiguous chunk.
-mlkd_status choose_grid(mlkd_context *ctx, int mode, bool coupled, int nbins, uint64_t count,
-                        int *grid, unsigned long long *ppw, int background)
+// Grid of the pair kernel: enough warps for 32 pairs each, up to one full wave
+// of resident blocks, and each warp an equal contiguous range.  With k full
+// sets of 32 pairs per resident warp and a rest, equal ranges give every warp a
+// last set that is mostly idle lanes.  For k = 1 the warps get 32 pairs each
+// instead and the rest goes to blocks of a second, partial wave, which start
+// as the first ones end (FP32 level 8 of the periodic problem, a rest of 0.02 /
+// 0.5 / 0.95 sets: 0.353 -> 0.241, 0.390 -> 0.313, 0.512 -> 0.401 ms; FP64 1.22 ->
+// 1.01, 1.36 -> 1.25, 1.83 -> 1.47; B1 level 10 0.89 -> 0.74, 1.04 -> 0.85, 1.49 ->
+// 1.02).  For larger k lanes that end early take the next pairs, which is worth
+// more than the rest (k = 2, rest 0.02: 0.52 ms, 0.56 in two waves), unless all
+// pairs have the same number of events, one in every step: there the ranges
+// are multiples of 32 up to k = 6 (level 4 at eps = 1e-3, k = 2: 0.163 -> 0.121 ms,
+// k = 6: 0.362 -> 0.341).
+mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, const PairLaunch &P, int *grid,
+                        unsigned long long *ppw)
 {
     KernelInfo info;
-    if (pair_kernel_info(mode, coupled, nbins, &info, background) != cudaSuccess) return MLKD_ECUDA;
-    const int per_sm = std::max(1, info.blocks_per_sm);
-    const long long wave = std::min<long long>((long long)ctx->sm_count * per_sm, kMaxBlocks);
-    const unsigned long long warps_needed = (count + 31) / 32;
-    const unsigned long long blocks_needed = (warps_needed + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    const long long g = (long long)std::min<unsigned long long>(blocks_needed, (unsigned long long)wave);
-    *grid = (int)std::max<long long>(1, g);
+    if (pair_kernel_info(mode, coupled, P.nbins, &info, P.background) != cudaSuccess) return MLKD_ECUDA;
+    const unsigned long long count = P.n_pairs;
+    const long long wave = std::min<long long>((long long)sm_count * std::max(1, info.blocks_per_sm), max_blocks);
+    const unsigned long long per_block = 32ull * kWarpsPerBlock;
+    const unsigned long long full = per_block * (unsigned long long)wave;
+    unsigned long long g = std::min<unsigned long long>((count + per_block - 1) / per_block, (unsigned long long)wave);
+    const unsigned long long k = count / full;
+    // fewer than half a step without a collision is expected per pair
+    const bool equal = (double)P.n * std::exp(-P.R * P.dt) < 0.5;
+    if (k == 1 || (equal && k >= 1 && k <= 6 && (double)(count % full) < 0.9 * (double)full)) {
+        const unsigned long long more = (count + k * per_block - 1) / (k * per_block);
+        if (more <= (unsigned long long)max_blocks) g = more;
+    }
+    *grid = (int)std::max<unsigned long long>(1, g);
     const unsigned long long warps = (unsigned long long)(*grid) * kWarpsPerBlock;
     *ppw = (count + warps - 1) / warps;
     return MLKD_OK;
@@ -299,7 +317,7 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     fill_launch(p, d, level, first, count, &P);
     int grid = 1;
     unsigned long long ppw = 0;
-    mlkd_status st = choose_grid(ctx, d.mode, level > 0, p->nbins, count, &grid, &ppw, d.background);
+    mlkd_status st = choose_grid(ctx->sm_count, kMaxBlocks, d.mode, level > 0, P, &grid, &ppw);
     if (st != MLKD_OK) return st;
     P.pairs_per_warp = ppw;
     P.partials = partials;
@@ -1047,19 +1065,11 @@ extern "C" mlkd_status mlkd_run_level_noalloc(const mlkd_problem *problem, int l
     cudaStream_t s = (cudaStream_t)stream;
     int sms = 0;
     MLKD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
-    KernelInfo info;
-    MLKD_CUDA(pair_kernel_info(d.mode, level > 0, problem->nbins, &info, d.background));
-    const long long wave = std::min<long long>((long long)sms * std::max(1, info.blocks_per_sm),
-                                               MLKD_NOALLOC_MAX_BLOCKS);
-    const unsigned long long warps_needed = (n_pairs + 31) / 32;
-    const unsigned long long blocks_needed = (warps_needed + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    const int grid = (int)std::max<long long>(
-        1, (long long)std::min<unsigned long long>(blocks_needed, (unsigned long long)wave));
-    const unsigned long long warps = (unsigned long long)grid * kWarpsPerBlock;
-
     PairLaunch P;
     fill_launch(problem, d, level, first_pair, n_pairs, &P);
-    P.pairs_per_warp = (n_pairs + warps - 1) / warps;
+    int grid = 1;
+    st = choose_grid(sms, MLKD_NOALLOC_MAX_BLOCKS, d.mode, level > 0, P, &grid, &P.pairs_per_warp);
+    if (st != MLKD_OK) return st;
     P.partials = (double *)scratch;
     P.partial_rows = MLKD_NOALLOC_MAX_BLOCKS;
     P.hist = problem->nbins > 0 ? (unsigned long long *)(scratch + kNoAllocHistOffset) : nullptr;
