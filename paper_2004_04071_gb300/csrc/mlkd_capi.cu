@@ -235,7 +235,9 @@ namespace {
 // Grid of the pair kernel: enough warps for 32 pairs each, up to one full wave
 // of resident blocks, and each warp an equal contiguous range.  With k full
 // sets of 32 pairs per resident warp and a rest, equal ranges give every warp a
-// last set that is mostly idle lanes.  For k = 1 the warps get 32 pairs each
+// last set that is mostly idle lanes.  For k = 1 and pairs of at least 8 events
+// (with two the second wave's starts cost more: FP64 level 1 of the free-space
+// problem, 1.95 sets, 77 -> 104 us) the warps get 32 pairs each
 // instead and the rest goes to blocks of a second, partial wave, which start
 // as the first ones end (FP32 level 8 of the periodic problem, a rest of 0.02 /
 // 0.5 / 0.95 sets: 0.353 -> 0.241, 0.390 -> 0.313, 0.512 -> 0.401 ms; FP64 1.22 ->
@@ -243,8 +245,9 @@ namespace {
 // 1.02).  For larger k lanes that end early take the next pairs, which is worth
 // more than the rest (k = 2, rest 0.02: 0.52 ms, 0.56 in two waves), unless all
 // pairs have the same number of events, one in every step: there the ranges
-// are multiples of 32 up to k = 6 (level 4 at eps = 1e-3, k = 2: 0.163 -> 0.121 ms,
-// k = 6: 0.362 -> 0.341).
+// of FP32 launches are multiples of 32 up to k = 6 (level 4 at eps = 1e-3, k = 2:
+// 0.163 -> 0.121 ms, k = 6: 0.362 -> 0.341; FP64 launches lose, 0.52 -> 0.63 ms for
+// 500 000 pairs of level 3).
 mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, const PairLaunch &P, int *grid,
                         unsigned long long *ppw)
 {
@@ -256,9 +259,10 @@ mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, co
     const unsigned long long full = per_block * (unsigned long long)wave;
     unsigned long long g = std::min<unsigned long long>((count + per_block - 1) / per_block, (unsigned long long)wave);
     const unsigned long long k = count / full;
-    // fewer than half a step without a collision is expected per pair
-    const bool equal = (double)P.n * std::exp(-P.R * P.dt) < 0.5;
-    if (k == 1 || (equal && k >= 1 && k <= 6 && (double)(count % full) < 0.9 * (double)full)) {
+    // events expected per pair; fewer than half a step without a collision
+    const double events = -(double)P.n * std::expm1(-P.R * P.dt);
+    const bool equal = mode != kModeFP64 && mode != kModeFP64U24 && (double)P.n * std::exp(-P.R * P.dt) < 0.5;
+    if (events >= 8.0 && (k == 1 || (equal && k >= 1 && k <= 6 && (double)(count % full) < 0.9 * (double)full))) {
         const unsigned long long more = (count + k * per_block - 1) / (k * per_block);
         if (more <= (unsigned long long)max_blocks) g = more;
     }
