@@ -62,11 +62,14 @@ template <typename Real> struct BgParams {
     Real lo, hi, inv_h;
 };
 
-// Parameters of one pair-kernel launch (passed by value as __grid_constant__).
-// Idle lanes a warp of the pair kernels gathers before it sums their finished
-// pairs and starts new ones in one pass (the batched form can override it).
-constexpr int kRefillMin = 8;
+// Idle lanes a warp of the per-level kernel gathers before it sums their
+// finished pairs and starts new ones in one pass.  Homogeneous events: 6 (2^20
+// FP32 pairs of level 8 of the periodic problem 1.27 ms, 1.30 with 8, 1.28 with 4,
+// 1.34 with 2, 1.43 with 12; FP64 9.12, 9.40, 9.17, 9.51, 10.3).  The
+// heterogeneous event is longer against a start: 8 (4 loses 1 %).
+template <int PHYS> constexpr int kRefillMin = PHYS == 1 ? 8 : 6;
 
+// Parameters of one pair-kernel launch (passed by value as __grid_constant__).
 struct PairLaunch {
     double R, mu, sigma, dt;   // background and fine step of this level
     double lo, hi, h;          // histogram range [lo, hi) and bin width

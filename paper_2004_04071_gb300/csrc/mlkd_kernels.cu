@@ -154,7 +154,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
         // the whole warp) can be summed and restarted from the warp's chunk
         // in one pass.
         const unsigned idle = __ballot_sync(kFullMask, !active);
-        if (idle != 0u && (__popc(idle) >= kRefillMin || idle == kFullMask)) {
+        if (idle != 0u && (__popc(idle) >= kRefillMin<PHYS> || idle == kFullMask)) {
             if (done) finish_pair();
             if (next < w_end) {
                 const unsigned rank = __popc(idle & ((1u << lane) - 1u));
