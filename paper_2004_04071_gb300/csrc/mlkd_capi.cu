@@ -34,13 +34,14 @@ Layout arena_layout()
         }
         return at;
     };
-    // one scratch slot (block partials, level sums, histogram) per level, so
-    // that the levels of a round can run at the same time
+    // one scratch slot (block partials, arrival counter) per level, so that the
+    // levels of a round can run at the same time
     L.partials = place((size_t)MLKD_MAX_LEVELS * kMaxBlocks * kPartialWords * sizeof(double));
-    L.tmp_stats = place(MLKD_MAX_LEVELS * sizeof(DevLevelStats));
+    L.out = place(kOutHist + 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_stats = place(MLKD_MAX_LEVELS * sizeof(DevLevelStats));
-    L.tmp_hist = place((size_t)MLKD_MAX_LEVELS * 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
+    L.tmp_hist = place(3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_hist = place((size_t)MLKD_MAX_LEVELS * 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
+    L.arrived = place(MLKD_MAX_LEVELS * sizeof(unsigned));
     L.control = place(sizeof(DevControl));
     L.total = off;
     return L;
@@ -307,7 +308,8 @@ mlkd_status mlkd::harvest_timing(mlkd_context *ctx)
 
 namespace {
 
-// Enqueues one level run: pair kernel + fixed-order finalize (+ accumulation).
+// Enqueues one level run: the pair kernel, whose last block sums the block rows
+// (and accumulates them).
 mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derived &d, int level,
                           uint64_t first, uint64_t count, cudaStream_t stream,
                           bool accumulate, double *dxf, double *dxc, int32_t *dkf, int32_t *dkc,
@@ -315,8 +317,6 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
 {
     // this launch's scratch slot: concurrent launches use different slots
     double *partials = ctx->partials + (size_t)slot * kMaxBlocks * kPartialWords;
-    DevLevelStats *tmp_stats = ctx->tmp_stats + slot;
-    unsigned long long *tmp_hist = ctx->tmp_hist + (size_t)slot * 3 * MLKD_MAX_BINS;
     PairLaunch P;
     fill_launch(p, d, level, first, count, &P);
     int grid = 1;
@@ -326,13 +326,21 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.pairs_per_warp = ppw;
     P.partials = partials;
     P.partial_rows = kMaxBlocks;
-    P.hist = p->nbins > 0 ? tmp_hist : nullptr;
+    P.arrived = ctx->arrived + slot;
+    if (accumulate) {
+        P.acc = ctx->acc_stats + level;
+        if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
+    } else {
+        P.stats = (DevLevelStats *)ctx->out;
+        if (p->nbins > 0) {
+            P.hist = ctx->tmp_hist;
+            P.hist_out = (unsigned long long *)(ctx->out + kOutHist);
+        }
+    }
     P.dbg_xf = dxf;
     P.dbg_xc = dxc;
     P.dbg_kf = dkf;
     P.dbg_kc = dkc;
-    if (p->nbins > 0)
-        MLKD_CUDA(cudaMemsetAsync(tmp_hist, 0, 3 * (size_t)p->nbins * sizeof(unsigned long long), stream));
     const bool timed = ctx->timing && ctx->events_made;
     if (timed && ctx->pending == kTimingRing) {
         mlkd_status st2 = harvest_timing(ctx);
@@ -341,14 +349,18 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     if (timed) MLKD_CUDA(cudaEventRecord(ctx->ev_start[ctx->pending], stream));
     MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, stream));
     if (timed) MLKD_CUDA(cudaEventRecord(ctx->ev_stop[ctx->pending++], stream));
-    MLKD_CUDA(launch_finalize(partials, grid, (long long)count, tmp_stats,
-                              accumulate ? ctx->acc_stats + level : nullptr, stream));
-    ++ctx->other_launches;
-    if (accumulate && p->nbins > 0) {
-        MLKD_CUDA(launch_hist_accumulate(tmp_hist, ctx->acc_hist + (size_t)level * 3 * p->nbins,
-                                         3 * p->nbins, stream));
-        ++ctx->other_launches;
+    return MLKD_OK;
+}
+
+// Zeroes the histogram scratch and the arrival counters, on the stream of the
+// first call and after a call that failed.  Every launch leaves them zero.
+mlkd_status ensure_clean(mlkd_context *ctx, cudaStream_t s)
+{
+    if (!ctx->clean) {
+        MLKD_CUDA(cudaMemsetAsync(ctx->tmp_hist, 0, 3 * MLKD_MAX_BINS * sizeof(unsigned long long), s));
+        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * sizeof(unsigned), s));
     }
+    ctx->clean = false;            // until the call has synchronised
     return MLKD_OK;
 }
 
@@ -445,7 +457,9 @@ mlkd_status mlkd_context_create(int device, void *arena, size_t arena_bytes, mlk
     c->arena_bytes = arena_bytes;
     c->L = L;
     c->partials = (double *)(c->arena + L.partials);
-    c->tmp_stats = (DevLevelStats *)(c->arena + L.tmp_stats);
+    c->out = c->arena + L.out;
+    c->arrived = (unsigned *)(c->arena + L.arrived);
+    c->clean = false;
     c->acc_stats = (DevLevelStats *)(c->arena + L.acc_stats);
     c->tmp_hist = (unsigned long long *)(c->arena + L.tmp_hist);
     c->acc_hist = (unsigned long long *)(c->arena + L.acc_hist);
@@ -698,16 +712,20 @@ mlkd_status mlkd_run_level(mlkd_context *ctx, const mlkd_problem *problem, int l
         if (hist_out && problem->nbins > 0) std::memset(hist_out, 0, 3 * (size_t)problem->nbins * sizeof(uint64_t));
         return MLKD_OK;
     }
-    mlkd_status st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false,
-                                   nullptr, nullptr, nullptr, nullptr);
+    mlkd_status st = ensure_clean(ctx, s);
     if (st != MLKD_OK) return st;
-    DevLevelStats hs;
-    MLKD_CUDA(cudaMemcpyAsync(&hs, ctx->tmp_stats, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    if (hist_out && problem->nbins > 0)
-        MLKD_CUDA(cudaMemcpyAsync(hist_out, ctx->tmp_hist, 3 * (size_t)problem->nbins * sizeof(uint64_t),
-                                  cudaMemcpyDeviceToHost, s));
+    st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false, nullptr, nullptr, nullptr, nullptr);
+    if (st != MLKD_OK) return st;
+    // sums and histogram in one copy
+    unsigned char buf[kOutHist + 3 * MLKD_MAX_BINS * sizeof(uint64_t)];
+    const size_t nh = hist_out ? 3 * (size_t)problem->nbins * sizeof(uint64_t) : 0;
+    MLKD_CUDA(cudaMemcpyAsync(buf, ctx->out, nh ? kOutHist + nh : sizeof(DevLevelStats), cudaMemcpyDeviceToHost, s));
     MLKD_CUDA(cudaStreamSynchronize(s));
+    ctx->clean = true;
+    DevLevelStats hs;
+    std::memcpy(&hs, buf, sizeof(hs));
     to_host_stats(hs, out);
+    if (nh) std::memcpy(hist_out, buf + kOutHist, nh);
     st = harvest_timing(ctx);
     if (st == MLKD_OK) st = device_checks();
     return st != MLKD_OK ? st : guards_check(ctx->arena, ctx->L.guard, ctx->L.n_guard);
@@ -725,10 +743,12 @@ mlkd_status mlkd_debug_pairs(mlkd_context *ctx, const mlkd_problem *problem, int
     cudaStream_t s = (cudaStream_t)stream;
     MLKD_CUDA(cudaSetDevice(ctx->device));
     if (n_pairs == 0) return MLKD_OK;
-    mlkd_status st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false, xf, xc,
-                                   kf, kc);
+    mlkd_status st = ensure_clean(ctx, s);
+    if (st != MLKD_OK) return st;
+    st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false, xf, xc, kf, kc);
     if (st != MLKD_OK) return st;
     MLKD_CUDA(cudaStreamSynchronize(s));
+    ctx->clean = true;
     return harvest_timing(ctx);
 }
 
@@ -789,6 +809,10 @@ static mlkd_status estimate_impl(mlkd_context *ctx, const mlkd_problem *problem,
     MLKD_CUDA(cudaMemsetAsync(ctx->acc_stats, 0, nl * sizeof(DevLevelStats), s));
     if (nb > 0)
         MLKD_CUDA(cudaMemsetAsync(ctx->acc_hist, 0, (size_t)nl * 3 * nb * sizeof(unsigned long long), s));
+    {
+        const mlkd_status cs = ensure_clean(ctx, s);
+        if (cs != MLKD_OK) return cs;
+    }
     long long have[MLKD_MAX_LEVELS] = {0};
     const int density = problem->qoi == MLKD_QOI_DENSITY ? 1 : 0;
     DevControl ctl;
@@ -906,6 +930,7 @@ static mlkd_status estimate_impl(mlkd_context *ctx, const mlkd_problem *problem,
             for (int b = 0; b < nb; ++b) dens[b] /= d.h;
     }
     MLKD_CUDA(cudaStreamSynchronize(s));
+    ctx->clean = true;
     out->estimate = ctl.estimate;
     out->variance = ctl.variance;
     out->n_levels = nl;
@@ -978,7 +1003,10 @@ constexpr size_t kNoAllocStatsOffset = (size_t)MLKD_NOALLOC_MAX_BLOCKS * kPartia
 constexpr size_t kNoAllocHistOffset = kNoAllocStatsOffset + 256;
 constexpr size_t kNoAllocBytes = kNoAllocHistOffset + 3 * (size_t)MLKD_NOALLOC_MAX_BINS * sizeof(unsigned long long);
 static_assert(kNoAllocBytes == (size_t)MLKD_NOALLOC_SCRATCH_BYTES, "scratch size mismatch");
-static_assert(sizeof(DevLevelStats) <= 256, "level stats exceed their scratch slot");
+// the arrival counter shares the level sums' slot (zero when the module is
+// loaded, and after every launch)
+constexpr size_t kNoAllocArrivedOffset = kNoAllocStatsOffset + 128;
+static_assert(sizeof(DevLevelStats) <= 128, "level stats exceed their scratch slot");
 
 }  // namespace
 
@@ -1077,17 +1105,20 @@ extern "C" mlkd_status mlkd_run_level_noalloc(const mlkd_problem *problem, int l
     P.partials = (double *)scratch;
     P.partial_rows = MLKD_NOALLOC_MAX_BLOCKS;
     P.hist = problem->nbins > 0 ? (unsigned long long *)(scratch + kNoAllocHistOffset) : nullptr;
-    DevLevelStats *dstats = (DevLevelStats *)(scratch + kNoAllocStatsOffset);
+    P.stats = (DevLevelStats *)(scratch + kNoAllocStatsOffset);
+    P.arrived = (unsigned *)(scratch + kNoAllocArrivedOffset);
     if (problem->nbins > 0)   // counters keep the previous call's values
         MLKD_CUDA(cudaMemsetAsync(P.hist, 0, 3 * (size_t)problem->nbins * sizeof(unsigned long long), s));
     MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, s));
-    MLKD_CUDA(launch_finalize(P.partials, grid, (long long)n_pairs, dstats, nullptr, s));
-    DevLevelStats hs;
-    MLKD_CUDA(cudaMemcpyAsync(&hs, dstats, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    if (hist_out && problem->nbins > 0)
-        MLKD_CUDA(cudaMemcpyAsync(hist_out, P.hist, 3 * (size_t)problem->nbins * sizeof(uint64_t),
-                                  cudaMemcpyDeviceToHost, s));
+    // sums and histogram lie one behind the other: one copy
+    unsigned char buf[256 + 3 * MLKD_NOALLOC_MAX_BINS * sizeof(uint64_t)];
+    const size_t nh = hist_out ? 3 * (size_t)problem->nbins * sizeof(uint64_t) : 0;
+    MLKD_CUDA(cudaMemcpyAsync(buf, scratch + kNoAllocStatsOffset, nh ? 256 + nh : sizeof(DevLevelStats),
+                              cudaMemcpyDeviceToHost, s));
     MLKD_CUDA(cudaStreamSynchronize(s));
+    DevLevelStats hs;
+    std::memcpy(&hs, buf, sizeof(hs));
+    if (nh) std::memcpy(hist_out, buf + 256, nh);
     to_host_stats(hs, out);
     return MLKD_OK;
 }

@@ -30,6 +30,7 @@ constexpr size_t kAlign = 256;
 constexpr uint32_t kWeylA = 0x9E3779B9u;         // Philox key increments (SC'11)
 constexpr uint32_t kWeylB = 0xBB67AE85u;
 constexpr int kTimingRing = 64;
+constexpr size_t kOutHist = 256;                  // offset of a call's histogram behind its sums
 
 // Canary bytes after each arena region in the debug build (MLKD_CHECKS):
 // written when the region is set up, compared after each synchronising call.
@@ -43,7 +44,7 @@ constexpr int kMaxGuards = 16;
 
 // Arena layout of the base workspace (offsets in bytes).
 struct Layout {
-    size_t partials, tmp_stats, acc_stats, tmp_hist, acc_hist, control, total;
+    size_t partials, out, acc_stats, tmp_hist, acc_hist, arrived, control, total;
     size_t guard[kMaxGuards];    // canary offsets (debug build)
     int n_guard;
 };
@@ -103,8 +104,11 @@ struct mlkd_context {
     size_t arena_bytes;
     mlkd::Layout L;
     double *partials;
-    mlkd::DevLevelStats *tmp_stats, *acc_stats;
+    char *out;                            // a call's sums and, kOutHist bytes on, its histogram
+    mlkd::DevLevelStats *acc_stats;
     unsigned long long *tmp_hist, *acc_hist;
+    unsigned *arrived;                    // per scratch slot: blocks done of the launch in flight
+    bool clean;                           // tmp_hist and arrived are zero (every launch leaves them so)
     mlkd::DevControl *control;
     mlkd::BatchCache *batch;    // lazily created by the batched form
     mlkd::Server *server;       // running serving form, or null

