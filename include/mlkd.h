@@ -341,7 +341,7 @@ MLKD_API mlkd_status mlkd_debug_transforms(const uint32_t *words, uint64_t n, fl
 typedef struct {
     uint64_t launches;       /* pair-kernel launches timed                      */
     double pair_kernel_ms;   /* their summed device time                        */
-    uint64_t other_launches; /* finalize / controller / histogram launches      */
+    uint64_t other_launches; /* controller and other launches                    */
 } mlkd_kernel_timing;
 
 /* Turns the pair-kernel timing on (enable != 0) or off. */

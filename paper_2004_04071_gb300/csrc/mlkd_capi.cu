@@ -2,6 +2,7 @@
 // context over a caller-owned device arena, and the host side of the
 // per-level run and of the adaptive MLMC estimate (Sec. 4.1).
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -41,7 +42,7 @@ Layout arena_layout()
     L.acc_stats = place(MLKD_MAX_LEVELS * sizeof(DevLevelStats));
     L.tmp_hist = place(3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_hist = place((size_t)MLKD_MAX_LEVELS * 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
-    L.arrived = place(MLKD_MAX_LEVELS * sizeof(unsigned));
+    L.arrived = place(MLKD_MAX_LEVELS * sizeof(unsigned long long));
     L.control = place(sizeof(DevControl));
     L.total = off;
     return L;
@@ -169,7 +170,9 @@ namespace mlkd {
 void fill_launch(const mlkd_problem *p, const Derived &d, int j, uint64_t first, uint64_t count,
                  PairLaunch *P)
 {
+    static std::atomic<unsigned long long> last_ticket{0};
     std::memset(P, 0, sizeof(*P));
+    P->ticket = ++last_ticket;
     const int level = d.lev[j];                  // fine level of estimator level j
     const long long Ml = ipow(p->M, level);
     P->R = d.R;
@@ -353,12 +356,13 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
 }
 
 // Zeroes the histogram scratch and the arrival counters, on the stream of the
-// first call and after a call that failed.  Every launch leaves them zero.
+// first call and after a call that failed.  Every launch leaves the histogram
+// zero, and the counters below the next ticket.
 mlkd_status ensure_clean(mlkd_context *ctx, cudaStream_t s)
 {
     if (!ctx->clean) {
         MLKD_CUDA(cudaMemsetAsync(ctx->tmp_hist, 0, 3 * MLKD_MAX_BINS * sizeof(unsigned long long), s));
-        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * sizeof(unsigned), s));
+        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * sizeof(unsigned long long), s));
     }
     ctx->clean = false;            // until the call has synchronised
     return MLKD_OK;
@@ -458,7 +462,7 @@ mlkd_status mlkd_context_create(int device, void *arena, size_t arena_bytes, mlk
     c->L = L;
     c->partials = (double *)(c->arena + L.partials);
     c->out = c->arena + L.out;
-    c->arrived = (unsigned *)(c->arena + L.arrived);
+    c->arrived = (unsigned long long *)(c->arena + L.arrived);
     c->clean = false;
     c->acc_stats = (DevLevelStats *)(c->arena + L.acc_stats);
     c->tmp_hist = (unsigned long long *)(c->arena + L.tmp_hist);
@@ -994,7 +998,7 @@ mlkd_status mlkd_estimate_sequence(mlkd_context *ctx, const mlkd_problem *proble
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Allocation-free entry point: the same pair kernel and finalize, with their
+// Allocation-free entry point: the same pair kernel, with its
 // scratch in a file-scope device array instead of a caller arena.
 // ---------------------------------------------------------------------------
 namespace {
@@ -1004,7 +1008,7 @@ constexpr size_t kNoAllocHistOffset = kNoAllocStatsOffset + 256;
 constexpr size_t kNoAllocBytes = kNoAllocHistOffset + 3 * (size_t)MLKD_NOALLOC_MAX_BINS * sizeof(unsigned long long);
 static_assert(kNoAllocBytes == (size_t)MLKD_NOALLOC_SCRATCH_BYTES, "scratch size mismatch");
 // the arrival counter shares the level sums' slot (zero when the module is
-// loaded, and after every launch)
+// loaded; a launch counts from its own ticket on)
 constexpr size_t kNoAllocArrivedOffset = kNoAllocStatsOffset + 128;
 static_assert(sizeof(DevLevelStats) <= 128, "level stats exceed their scratch slot");
 
@@ -1106,7 +1110,7 @@ extern "C" mlkd_status mlkd_run_level_noalloc(const mlkd_problem *problem, int l
     P.partial_rows = MLKD_NOALLOC_MAX_BLOCKS;
     P.hist = problem->nbins > 0 ? (unsigned long long *)(scratch + kNoAllocHistOffset) : nullptr;
     P.stats = (DevLevelStats *)(scratch + kNoAllocStatsOffset);
-    P.arrived = (unsigned *)(scratch + kNoAllocArrivedOffset);
+    P.arrived = (unsigned long long *)(scratch + kNoAllocArrivedOffset);
     if (problem->nbins > 0)   // counters keep the previous call's values
         MLKD_CUDA(cudaMemsetAsync(P.hist, 0, 3 * (size_t)problem->nbins * sizeof(unsigned long long), s));
     MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, s));

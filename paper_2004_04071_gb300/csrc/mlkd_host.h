@@ -26,6 +26,7 @@ struct NvtxRange {
 };
 
 constexpr int kMaxBlocks = 4096;                  // grid cap of the pair kernel
+static_assert(kMaxBlocks < 1 << kTicketShift, "an arrival counter counts every block of a grid");
 constexpr size_t kAlign = 256;
 constexpr uint32_t kWeylA = 0x9E3779B9u;         // Philox key increments (SC'11)
 constexpr uint32_t kWeylB = 0xBB67AE85u;
@@ -107,8 +108,8 @@ struct mlkd_context {
     char *out;                            // a call's sums and, kOutHist bytes on, its histogram
     mlkd::DevLevelStats *acc_stats;
     unsigned long long *tmp_hist, *acc_hist;
-    unsigned *arrived;                    // per scratch slot: blocks done of the launch in flight
-    bool clean;                           // tmp_hist and arrived are zero (every launch leaves them so)
+    unsigned long long *arrived;          // per scratch slot: blocks done of the launch in flight
+    bool clean;                           // tmp_hist is zero (every launch leaves it so)
     mlkd::DevControl *control;
     mlkd::BatchCache *batch;    // lazily created by the batched form
     mlkd::Server *server;       // running serving form, or null

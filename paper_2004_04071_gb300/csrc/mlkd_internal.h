@@ -91,12 +91,18 @@ struct PairLaunch {
     double *partials;                  // [gridDim.x][kPartialWords]
     int32_t partial_rows;              // rows the partials buffer holds (>= gridDim.x)
     unsigned long long *hist;          // [3][nbins] fine, coarse, both counters to add to; or null
-    unsigned *arrived;                 // blocks done (0 between launches)
+    unsigned long long *arrived;       // ticket << kTicketShift | blocks of that launch done
+    unsigned long long ticket;         // this launch, numbered upwards in a process
     DevLevelStats *stats, *acc;        // the launch's sums go to *stats and are added to *acc (or null)
     unsigned long long *hist_out;      // hist is moved here and zeroed (or null: left in hist)
     double *dbg_xf, *dbg_xc;           // optional per-pair outputs
     int32_t *dbg_kf, *dbg_kc;
 };
+
+// Below the ticket in an arrival counter: room for any grid.  A launch's first
+// block raises the counter to its own ticket, so nothing an earlier launch left
+// there (calls that raced on one scratch buffer, say) is counted.
+constexpr int kTicketShift = 13;
 
 struct KernelInfo {
     int blocks_per_sm;
