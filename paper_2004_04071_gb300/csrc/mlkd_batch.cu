@@ -52,8 +52,10 @@ constexpr int kPublishSpins = 1 << 22;           // bounded wait for earlier res
 constexpr double kSmallRoundEvents = 2e8;        // predicted KD events of a round that goes first (about 2 ms)
 constexpr int kWarpPairEvents = 1024;            // events per pair from which a pair runs on a whole warp
 constexpr int kSliceWaitIters = 128;              // slices shorter than this (about 0.1 ms) are over before a wait pays
-constexpr int kSliceIdleSpins = 20;               // the same in a sliced launch: about 1 ms
-constexpr int kIdleSpins = 4096;                 // bounded wait for new work: sleeps of up to 64 us, about 0.25 s
+constexpr int kSliceIdleSpins = 256;              // bounded wait for new work in a sliced launch: sleeps of up to 4 us, about 1 ms
+constexpr int kSliceIdleShift = 2;                // (a slice ends with its last waiting warp: sleeps of 64 us cost 5 %)
+constexpr int kIdleSpins = 4096;                 // the same in an unbounded launch: sleeps of up to 64 us, about 0.25 s
+constexpr int kIdleShift = 6;
 
 struct ReqDesc {
     BgParams<double> bd[kBL];
@@ -940,7 +942,7 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
             // while some warp is at work; the next slice picks up what is published
             // later.  (When such a warp left at once, the one that completed
             // a round worked alone on the next until its budget was spent: 8
-            // small FP64 requests in slices of 256 took 2.8 ms, now 1.6.)
+            // small FP64 requests in slices of 256 took 4.4 ms, now 2.4.)
             unsigned long long cn = 0;
             int got = 0;
             if (lane == 0) {
@@ -960,9 +962,10 @@ batch_pair_kernel(const __grid_constant__ BatchLaunch B)
                            idle >= idle_limit ||
                            (B.slice_iters > 0 && idle >= 2 && *(volatile int32_t *)&B.ctl->busy <= 0);
                 if (__shfl_sync(kFullMask, stop, 0)) break;
-                // back off to sleeps of 64 us, so that waiting warps take
+                // back off to the longest sleep, so that waiting warps take
                 // almost no issue slots from the warps still at work
-                __nanosleep(1000u << (idle < 6 ? idle : 6));
+                const int most = B.slice_iters > 0 ? kSliceIdleShift : kIdleShift;
+                __nanosleep(1000u << (idle < most ? idle : most));
                 continue;
             }
             idle = 0;
