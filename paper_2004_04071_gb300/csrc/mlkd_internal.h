@@ -62,12 +62,13 @@ template <typename Real> struct BgParams {
     Real lo, hi, inv_h;
 };
 
-// Idle lanes a warp of the per-level kernel gathers before it sums their
-// finished pairs and starts new ones in one pass.  Homogeneous events: 6 (2^20
-// FP32 pairs of level 8 of the periodic problem 1.27 ms, 1.30 with 8, 1.28 with 4,
-// 1.34 with 2, 1.43 with 12; FP64 9.12, 9.40, 9.17, 9.51, 10.3).  The
-// heterogeneous event is longer against a start: 8 (4 loses 1 %).
-template <int PHYS> constexpr int kRefillMin = PHYS == 1 ? 8 : 6;
+// Idle lanes a warp of the per-level kernel gathers before it takes up new
+// pairs.  Coupled homogeneous pairs, which are started and summed 32 at a time
+// (2^20 pairs of level 8 of the periodic problem): 2 (FP32 1.22 ms, 1.22 with 3,
+// 1.25 with 4, 1.26 with 6, 1.30 with 8; FP64 8.88, 9.00, 9.25, 9.48, 9.87).  The
+// others sum and start them there and then: 6, and 8 for the heterogeneous
+// event, which is longer against a start (4 loses 1 %).
+template <int PHYS, bool COUPLED> constexpr int kRefillMin = PHYS == 1 ? 8 : COUPLED ? 2 : 6;
 
 // Parameters of one pair-kernel launch (passed by value as __grid_constant__).
 struct PairLaunch {

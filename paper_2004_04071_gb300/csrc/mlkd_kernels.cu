@@ -35,6 +35,24 @@ template <int PHYS> struct MinBlocks<double, PHYS> { static constexpr int value 
 template <typename Real, int PHYS> struct PhysState { typedef PairState<Real> type; };
 template <typename Real> struct PhysState<Real, 1> { typedef HetPairState<Real> type; };
 
+// Per warp: pairs started 32 at a time, and a ring of finished pairs that are
+// summed 32 at a time, so that neither path runs for only the few lanes that
+// fell idle together, and lanes wait less.  For coupled homogeneous pairs, with
+// a loop that holds nothing but the event (level 8 of the periodic problem,
+// 2^20 pairs: FP32 1.37 -> 1.21 ms, FP64 9.7 -> 8.9; 1000 pairs of level 10,
+// whose chains are all there is: 1.15 -> 0.87 ms, FP64 4.59 -> 4.42).  Uncoupled
+// pairs have so few events that the queues cost more than they save (5e6 paths
+// of level 0: FP32 0.18 ms without, 0.21 with them), and the heterogeneous
+// event is long enough (level 10 of B1: 2.39 and 2.43 ms).
+template <typename Real> struct StartedPairs {
+    Real x0[32], v0[32], q0[32];
+    int32_t off[32];                 // pair number - the first started one's
+};
+template <typename Real> struct FinishedPairs {
+    Real xf[64], xc[64];             // both paths at T
+    uint32_t kf[64], kc[64];         // fine and coarse events
+};
+
 // Run by the last block of a launch: the block rows in a fixed order into the
 // launch's sums (16 row groups of 8 words; lane and group sums in a fixed
 // tree), the histogram to its reader and its counters back to zero.  Folding
@@ -160,13 +178,16 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     unsigned long long next = w_begin;                 // warp-uniform
 
     bool active = false;        // the lane's pair has events left
-    bool done = false;          // the lane holds a finished pair not yet summed
     unsigned long long pair = 0;
+    bool done = false;          // the lane holds a finished pair not yet queued for summing
     typename PhysState<Real, PHYS>::type st;
     st.fresh = true;
-    // FP64: the running sums in shared memory, so that the event loop fits 64
-    // registers (8 blocks per SM)
-    constexpr bool kSharedSums = std::is_same<Real, double>::value;
+    // queues of started and finished pairs (see StartedPairs)
+    constexpr bool kQueues = COUPLED && PHYS == 0;
+    // Sums in shared memory with queues (they change once per 32 pairs) and in
+    // FP64, so that the event loop has the registers (FP32 coupled: 64, 8
+    // blocks per SM).
+    constexpr bool kSharedSums = kQueues || std::is_same<Real, double>::value;
     __shared__ LaneSums<MODE> s_sums[kSharedSums ? kThreads : 1];
     LaneSums<MODE> r_sums;
     LaneSums<MODE> &sums = kSharedSums ? s_sums[kSharedSums ? threadIdx.x : 0] : r_sums;
@@ -175,44 +196,159 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     mom.zero();
     ev_f_sum = 0;
     ev_c_sum = 0;
+    const unsigned lower = (1u << lane) - 1u;
 
-    // QoI, sums and histogram of the finished pair.
-    auto finish_pair = [&]() {
-        if constexpr (PHYS == 1)
-            het_pair_drift<Real>(st, H, COUPLED);
-        else
-            pair_drift<Real, CPL>(st, L, COUPLED);
-        add_pair_fk(mom, st.xf, st.xc, COUPLED, P.fkind);
-        ev_f_sum += st.k;
-        ev_c_sum += st.evc;
+    auto record = [&](unsigned long long pair, Real xf, Real xc, uint32_t kf, uint32_t kc) {
+        if (P.dbg_xf && MLKD_DCHECK(pair - P.first_pair < P.n_pairs)) {
+            const unsigned long long j = pair - P.first_pair;
+            P.dbg_xf[j] = (double)xf;
+            if (P.dbg_xc) P.dbg_xc[j] = COUPLED ? (double)xc : 0.0;
+            if (P.dbg_kf) P.dbg_kf[j] = (int32_t)kf;
+            if (P.dbg_kc) P.dbg_kc[j] = (int32_t)kc;
+        }
+    };
+    // QoI, sums and histogram of one finished pair.
+    auto account = [&](Real xf, Real xc, uint32_t kf, uint32_t kc) {
+        add_pair_fk(mom, xf, xc, COUPLED, P.fkind);
+        ev_f_sum += kf;
+        ev_c_sum += kc;
         if (nbins > 0) {
-            int bf = bins(st.xf);
+            int bf = bins(xf);
             if (!MLKD_DCHECK(bf < nbins)) bf = -1;
             if (bf >= 0) atomicAdd(&s_hist[bf], 1u);
             if (COUPLED) {
-                int bc = bins(st.xc);
+                int bc = bins(xc);
                 if (!MLKD_DCHECK(bc < nbins)) bc = -1;
                 if (bc >= 0) atomicAdd(&s_hist[nbins + bc], 1u);
                 if (bc >= 0 && bc == bf) atomicAdd(&s_hist[2 * nbins + bf], 1u);
             }
         }
-        if (P.dbg_xf && MLKD_DCHECK(pair - P.first_pair < P.n_pairs)) {
-            const unsigned long long j = pair - P.first_pair;
-            P.dbg_xf[j] = (double)st.xf;
-            if (P.dbg_xc) P.dbg_xc[j] = COUPLED ? (double)st.xc : 0.0;
-            if (P.dbg_kf) P.dbg_kf[j] = (int32_t)st.k;
-            if (P.dbg_kc) P.dbg_kc[j] = (int32_t)st.evc;
-        }
-        done = false;
     };
 
+    if constexpr (kQueues) {
+    // warp-uniform: started pairs taken and held, the number of the first of
+    // them, and the ring of finished pairs
+    __shared__ StartedPairs<Real> s_started[kWarpsPerBlock];
+    __shared__ FinishedPairs<Real> s_finished[kWarpsPerBlock];
+    StartedPairs<Real> &SP = s_started[threadIdx.x >> 5];
+    FinishedPairs<Real> &FP = s_finished[threadIdx.x >> 5];
+    unsigned long long sp_base = w_begin;
+    int sp_i = 0, sp_n = 0, fp_head = 0, fp_n = 0;
+    // Moves the lane's finished pair to T.
+    auto drift = [&]() {
+        pair_drift<Real, CPL>(st, L, COUPLED);
+        if (P.dbg_xf) record(((unsigned long long)(st.word2 ^ L.word2) << 32) | st.pair_lo, st.xf, st.xc, st.k, st.evc);
+    };
+    // Sums the first cnt queued pairs, one per lane.
+    auto sum_finished = [&](int cnt) {
+        __syncwarp();
+        if (lane < cnt) {
+            const int i = (fp_head + lane) & 63;
+            account(FP.xf[i], FP.xc[i], FP.kf[i], FP.kc[i]);
+        }
+        fp_head = (fp_head + cnt) & 63;
+        fp_n -= cnt;
+        __syncwarp();
+    };
+    // Queues the pairs of the lanes with f set, in lane order; fewer than 32
+    // are queued before and after.
+    auto queue_finished = [&](bool f, Real xf, Real xc, uint32_t kf, uint32_t kc) {
+        const unsigned m = __ballot_sync(kFullMask, f);
+        if (f) {
+            const int i = (fp_head + fp_n + __popc(m & lower)) & 63;
+            FP.xf[i] = xf;
+            FP.xc[i] = xc;
+            FP.kf[i] = kf;
+            FP.kc[i] = kc;
+        }
+        fp_n += __popc(m);
+        if (fp_n >= 32) sum_finished(32);
+    };
+    // Starts the next pairs of the warp's range, one per lane (with no started
+    // pair left).  A pair without a collision before T is finished at once.
+    auto start_pairs = [&]() {
+        const unsigned long long rest = w_end - next;
+        const int nav = rest < 32ull ? (int)rest : 32;
+        const unsigned long long p = next + (unsigned long long)lane;
+        const bool have = lane < nav;
+        Real x0 = Real(0), v0 = Real(0), q0 = Real(0);
+        bool dead = false;
+        if (have) {
+            pair_start_values<Real, RECIPE>(x0, v0, q0, p, L, P.keys);
+            if (P.init == 2) x0 = (Real)P.x0;
+            dead = !collides_before_T(L, q0);
+        }
+        const Real xT = dead ? straight_to_T<Real, PHYS>(x0, v0, L) : Real(0);
+        if (dead) record(p, xT, xT, 0u, 0u);
+        queue_finished(dead, xT, xT, 0u, 0u);
+        const bool live = have && !dead;
+        const unsigned lm = __ballot_sync(kFullMask, live);
+        __syncwarp();
+        if (live) {
+            const int i = __popc(lm & lower);
+            SP.x0[i] = x0;
+            SP.v0[i] = v0;
+            SP.q0[i] = q0;
+            SP.off[i] = lane;
+        }
+        sp_base = next;
+        sp_n = __popc(lm);
+        sp_i = 0;
+        next += (unsigned long long)nav;
+        __syncwarp();
+    };
+    unsigned idle = kFullMask;
+    int need = kRefillMin<PHYS, COUPLED>;          // idle lanes that end the event loop
+    for (;;) {
+        if (__any_sync(kFullMask, done)) {
+            if (done) drift();
+            queue_finished(done, st.xf, st.xc, st.k, st.evc);
+            done = false;
+        }
+        while (idle != 0u) {
+            if (sp_i == sp_n) {
+                if (next >= w_end) break;
+                start_pairs();
+                continue;
+            }
+            const int avail = sp_n - sp_i, rank = __popc(idle & lower);
+            if (!active && rank < avail) {
+                const int e = sp_i + rank;
+                pair_init<Real, CPL>(st, sp_base + (unsigned long long)SP.off[e], SP.x0[e], SP.v0[e], SP.q0[e], L,
+                                     COUPLED);
+                active = true;
+            }
+            sp_i += min(__popc(idle), avail);
+            idle = __ballot_sync(kFullMask, !active);
+        }
+        if (idle == kFullMask) break;
+        // with nothing left to hand out, the rest runs to its end
+        if (next >= w_end && sp_i == sp_n) need = 32;
+        do {
+            if (active && pair_event<Real, CPL, RECIPE>(st, L, P.keys, COUPLED)) {
+                active = false;
+                done = true;
+            }
+            idle = __ballot_sync(kFullMask, !active);
+        } while (__popc(idle) < need);
+    }
+    if (fp_n > 0) sum_finished(fp_n);
+    } else
     for (;;) {
         // Lanes whose pair reached T stay idle until kRefillMin of them (or
         // the whole warp) can be summed and restarted from the warp's chunk
         // in one pass.
         const unsigned idle = __ballot_sync(kFullMask, !active);
-        if (idle != 0u && (__popc(idle) >= kRefillMin<PHYS> || idle == kFullMask)) {
-            if (done) finish_pair();
+        if (idle != 0u && (__popc(idle) >= kRefillMin<PHYS, COUPLED> || idle == kFullMask)) {
+            if (done) {
+                if constexpr (PHYS == 1)
+                    het_pair_drift<Real>(st, H, COUPLED);
+                else
+                    pair_drift<Real, CPL>(st, L, COUPLED);
+                account(st.xf, COUPLED ? st.xc : Real(0), st.k, st.evc);
+                record(pair, st.xf, st.xc, st.k, st.evc);
+                done = false;
+            }
             if (next < w_end) {
                 const unsigned rank = __popc(idle & ((1u << lane) - 1u));
                 const unsigned long long cand = next + rank;
