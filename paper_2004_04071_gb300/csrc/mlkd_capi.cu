@@ -42,7 +42,7 @@ Layout arena_layout()
     L.acc_stats = place(MLKD_MAX_LEVELS * sizeof(DevLevelStats));
     L.tmp_hist = place(3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_hist = place((size_t)MLKD_MAX_LEVELS * 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
-    L.arrived = place(MLKD_MAX_LEVELS * sizeof(unsigned long long));
+    L.arrived = place(MLKD_MAX_LEVELS * kArrivals * sizeof(unsigned long long));
     L.control = place(sizeof(DevControl));
     L.total = off;
     return L;
@@ -329,7 +329,7 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.pairs_per_warp = ppw;
     P.partials = partials;
     P.partial_rows = kMaxBlocks;
-    P.arrived = ctx->arrived + slot;
+    P.arrived = ctx->arrived + (size_t)slot * kArrivals;
     if (accumulate) {
         P.acc = ctx->acc_stats + level;
         if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
@@ -362,7 +362,7 @@ mlkd_status ensure_clean(mlkd_context *ctx, cudaStream_t s)
 {
     if (!ctx->clean) {
         MLKD_CUDA(cudaMemsetAsync(ctx->tmp_hist, 0, 3 * MLKD_MAX_BINS * sizeof(unsigned long long), s));
-        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * sizeof(unsigned long long), s));
+        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * kArrivals * sizeof(unsigned long long), s));
     }
     ctx->clean = false;            // until the call has synchronised
     return MLKD_OK;
@@ -1007,10 +1007,11 @@ constexpr size_t kNoAllocStatsOffset = (size_t)MLKD_NOALLOC_MAX_BLOCKS * kPartia
 constexpr size_t kNoAllocHistOffset = kNoAllocStatsOffset + 256;
 constexpr size_t kNoAllocBytes = kNoAllocHistOffset + 3 * (size_t)MLKD_NOALLOC_MAX_BINS * sizeof(unsigned long long);
 static_assert(kNoAllocBytes == (size_t)MLKD_NOALLOC_SCRATCH_BYTES, "scratch size mismatch");
-// the arrival counter shares the level sums' slot (zero when the module is
+// the arrival counters share the level sums' slot (zero when the module is
 // loaded; a launch counts from its own ticket on)
 constexpr size_t kNoAllocArrivedOffset = kNoAllocStatsOffset + 128;
-static_assert(sizeof(DevLevelStats) <= 128, "level stats exceed their scratch slot");
+static_assert(sizeof(DevLevelStats) <= 128 && kArrivals * sizeof(unsigned long long) <= 128,
+              "level sums or arrival counters exceed their scratch slot");
 
 }  // namespace
 

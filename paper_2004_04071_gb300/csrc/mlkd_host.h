@@ -108,7 +108,7 @@ struct mlkd_context {
     char *out;                            // a call's sums and, kOutHist bytes on, its histogram
     mlkd::DevLevelStats *acc_stats;
     unsigned long long *tmp_hist, *acc_hist;
-    unsigned long long *arrived;          // per scratch slot: blocks done of the launch in flight
+    unsigned long long *arrived;          // per scratch slot: arrival counters of the launch in flight
     bool clean;                           // tmp_hist is zero (every launch leaves it so)
     mlkd::DevControl *control;
     mlkd::BatchCache *batch;    // lazily created by the batched form

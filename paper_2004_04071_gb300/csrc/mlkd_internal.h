@@ -92,7 +92,7 @@ struct PairLaunch {
     double *partials;                  // [gridDim.x][kPartialWords]
     int32_t partial_rows;              // rows the partials buffer holds (>= gridDim.x)
     unsigned long long *hist;          // [3][nbins] fine, coarse, both counters to add to; or null
-    unsigned long long *arrived;       // ticket << kTicketShift | blocks of that launch done
+    unsigned long long *arrived;       // [kArrivals], each ticket << kTicketShift | arrivals of that launch
     unsigned long long ticket;         // this launch, numbered upwards in a process
     DevLevelStats *stats, *acc;        // the launch's sums go to *stats and are added to *acc (or null)
     unsigned long long *hist_out;      // hist is moved here and zeroed (or null: left in hist)
@@ -104,6 +104,9 @@ struct PairLaunch {
 // block raises the counter to its own ticket, so nothing an earlier launch left
 // there (calls that raced on one scratch buffer, say) is counted.
 constexpr int kTicketShift = 13;
+// Arrival counters of a launch: of its groups of blocks, and of the blocks of each.
+constexpr int kArrivals = 16;
+constexpr int kOneGroup = 64;          // blocks that make one group
 
 struct KernelInfo {
     int blocks_per_sm;

@@ -53,31 +53,63 @@ template <typename Real> struct FinishedPairs {
     uint32_t kf[64], kc[64];         // fine and coarse events
 };
 
-// Run by the last block of a launch: the block rows in a fixed order into the
-// launch's sums (16 row groups of 8 words; lane and group sums in a fixed
-// tree), the histogram to its reader and its counters back to zero.  Folding
-// this into the pair kernel saves a launch, the clearing of the histogram and,
-// in an estimate, the launch that accumulated it, and one copy brings both
-// results to the host: 2000 FP64 pairs with 20 bins 88 -> 78 us, 300 paths with
-// 128 bins 50 -> 41 us, a small adaptive estimate with 64 bins 0.81 -> 0.70 ms.
-__device__ __noinline__ void finish_launch(const PairLaunch &P, double (*s_red)[kPartialWords])
+// Counts this block in; true in the launch's last of `blocks` to come here.
+__device__ __forceinline__ bool last_to_arrive(unsigned long long *counter, unsigned long long ticket, unsigned blocks)
 {
-    const int t = threadIdx.x, word = t & 7, groups = blockDim.x >> 3;
-    double v = 0.0;
-#pragma unroll 8
-    for (int b = t >> 3; b < (int)gridDim.x; b += groups)
-        v += __ldcg(&P.partials[(size_t)b * kPartialWords + word]);
-    v += __shfl_down_sync(kFullMask, v, 16);
-    v += __shfl_down_sync(kFullMask, v, 8);
-    if ((t & 31) < kPartialWords) s_red[t >> 5][word] = v;
-    __syncthreads();
-    if (t == 0) {
-        double w[kPartialWords];
+    atomicMax(counter, ticket << kTicketShift);
+    return (atomicAdd(counter, 1ull) & ((1ull << kTicketShift) - 1ull)) == blocks - 1u;
+}
+
+// Sums `count` block rows, `stride` rows apart, in a fixed order; every thread
+// of the block calls it.  Word j of the sum is left in s_red[0][j].
+__device__ __forceinline__ void sum_rows(double *rows, int stride, int count, double (*s_red)[kPartialWords])
+{
+    const int t = threadIdx.x, part = t & 3;
+    constexpr int kGroups = kThreads / 4, kAhead = 6;            // loads in flight per thread
+    double v0 = 0.0, v1 = 0.0;
+    for (int b0 = t >> 2; b0 < count; b0 += kGroups * kAhead) {
+        double2 r[kAhead];
 #pragma unroll
-        for (int j = 0; j < kPartialWords; ++j) {
-            w[j] = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) w[j] += s_red[k][j];
+        for (int j = 0; j < kAhead; ++j) {
+            const int b = b0 + j * kGroups;
+            r[j] = b < count ? __ldcg((const double2 *)(rows + (size_t)b * stride * kPartialWords) + part)
+                             : make_double2(0.0, 0.0);
         }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            v0 += r[j].x;
+            v1 += r[j].y;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off >= 4; off >>= 1) {
+        v0 += __shfl_down_sync(kFullMask, v0, off);
+        v1 += __shfl_down_sync(kFullMask, v1, off);
+    }
+    __syncthreads();
+    if ((t & 31) < 4) {
+        s_red[t >> 5][2 * part] = v0;
+        s_red[t >> 5][2 * part + 1] = v1;
+    }
+    __syncthreads();
+    if (t < kPartialWords) {
+        double w = s_red[0][t];
+        for (int k = 1; k < kWarpsPerBlock; ++k) w += s_red[k][t];
+        s_red[0][t] = w;                                         // no other thread reads it before the next barrier
+    }
+    __syncthreads();
+}
+
+// Run by the last block of a launch: the summed rows into the launch's sums, the
+// histogram to its reader and its counters back to zero.  Folding this into the
+// pair kernel saves a launch, the clearing of the histogram and, in an
+// estimate, the launch that accumulated it, and one copy brings both results
+// to the host: 2000 FP64 pairs with 20 bins 88 -> 78 us, 300 paths with 128 bins
+// 50 -> 41 us, a small adaptive estimate with 64 bins 0.81 -> 0.70 ms.
+__device__ __forceinline__ void finish_launch(const PairLaunch &P, const double *w)
+{
+    const int t = threadIdx.x;
+    if (t == 0) {
         DevLevelStats s;
         s.n = (long long)P.n_pairs;
         s.sy = w[0];
@@ -108,6 +140,40 @@ __device__ __noinline__ void finish_launch(const PairLaunch &P, double (*s_red)[
             P.hist[i] = 0ull;
         }
     }
+}
+
+// The end of a launch.  The last block to arrive sums the rows and finishes it.
+// Rows of large grids are first summed in groups, each by the group's last
+// block into its first row: one block alone would wait for the FP64 pipe and the
+// loads of all, and one counter for the arrivals of all (300 377 FP32 paths of
+// five events, 1216 blocks: a call takes 47 us, 71 without groups).
+__device__ __noinline__ void close_launch(const PairLaunch &P, double (*s_red)[kPartialWords])
+{
+    __shared__ bool s_last;
+    const int groups = (int)gridDim.x > kOneGroup ? kArrivals - 1 : 1;
+    const int per = ((int)gridDim.x + groups - 1) / groups;
+    const int group = (int)blockIdx.x / per, group_first = group * per;
+    const int group_size = min(per, (int)gridDim.x - group_first);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = last_to_arrive(P.arrived + 1 + group, P.ticket, (unsigned)group_size);
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double *first_row = P.partials + (size_t)group_first * kPartialWords;
+    sum_rows(first_row, 1, group_size, s_red);
+    if (groups > 1) {
+        const int used = ((int)gridDim.x + per - 1) / per;
+        if (threadIdx.x < kPartialWords) first_row[threadIdx.x] = s_red[0][threadIdx.x];
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = last_to_arrive(P.arrived, P.ticket, (unsigned)used);
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        sum_rows(P.partials, per, used, s_red);
+    }
+    finish_launch(P, s_red[0]);
 }
 
 template <typename Real, int MODE, bool COUPLED, int PHYS>
@@ -415,19 +481,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
         }
     }
 
-    // ---- the last block to arrive sums the rows and closes the launch ----
-    __shared__ bool s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        atomicMax(P.arrived, P.ticket << kTicketShift);
-        const unsigned long long done = atomicAdd(P.arrived, 1ull) & ((1ull << kTicketShift) - 1ull);
-        s_last = done == gridDim.x - 1u;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    finish_launch(P, s_red);
+    close_launch(P, s_red);
 }
 
 // ---------------------------------------------------------------------------

@@ -38,3 +38,25 @@ def test_calls_leave_nothing_behind(prec):
                             assert np.array_equal(r[k], hist[k]), (turn, n, nbins, k)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 2])
+def test_row_groups(prec):
+    """Grids around the sizes where block rows fall into groups: the sums are
+    those of the pairs."""
+    import paper_2004_04071_gb300 as mk
+    p = mk.make_problem(eps=0.5, T=0.5, dt0=0.1, M=2, L=1, qoi=0, init=0, precision=prec, seed=43)
+    ctx = mk.Context(0)
+    try:
+        whole = ctx.debug_pairs(p, 1, 0, 128 * 300)
+        for blocks in (1, 2, 15, 16, 63, 64, 65, 66, 75, 76, 90, 91, 225, 226, 300):
+            for n in (128 * blocks - 127, 128 * blocks):
+                xf, xc, kf, kc = (np.asarray(v[:n], np.float64) for v in whole)
+                for s in (ctx.run_level(p, 1, 0, n), mk.run_level_noalloc(p, 1, 0, n)):
+                    assert (s["n"], s["events_f"], s["events_c"]) == (n, int(kf.sum()), int(kc.sum()))
+                    # the square of a position in FP32 is rounded once (2^-24) over positive terms
+                    rel = 1e-12 if prec == 0 else 1e-6
+                    for k, x in (("sqf", xf), ("sqc", xc)):
+                        assert abs(s[k] - (x * x).sum()) <= rel * (x * x).sum(), (n, k)
+    finally:
+        ctx.close()
