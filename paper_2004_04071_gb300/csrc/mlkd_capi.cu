@@ -331,6 +331,7 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.partial_rows = kMaxBlocks;
     P.arrived = ctx->arrived + (size_t)slot * kArrivals;
     if (accumulate) {
+        MLKD_CUDA(prefer_shared_memory(d.mode, level > 0, d.background));
         P.acc = ctx->acc_stats + level;
         if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
     } else {

@@ -719,6 +719,12 @@ cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out,
     return e;
 }
 
+cudaError_t prefer_shared_memory(int mode, bool coupled, int background)
+{
+    return cudaFuncSetAttribute((const void *)pick(mode, coupled, background),
+                                cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid,
                                cudaStream_t stream)
 {
