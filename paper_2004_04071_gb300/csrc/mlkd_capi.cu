@@ -244,13 +244,13 @@ namespace {
 // problem, 1.95 sets, 77 -> 104 us) the warps get 32 pairs each
 // instead and the rest goes to blocks of a second, partial wave, which start
 // as the first ones end (FP32 level 8 of the periodic problem, a rest of 0.02 /
-// 0.5 / 0.95 sets: 0.353 -> 0.241, 0.390 -> 0.313, 0.512 -> 0.401 ms; FP64 1.22 ->
-// 1.01, 1.36 -> 1.25, 1.83 -> 1.47; B1 level 10 0.89 -> 0.74, 1.04 -> 0.85, 1.49 ->
-// 1.02).  For larger k lanes that end early take the next pairs, which is worth
-// more than the rest (k = 2, rest 0.02: 0.52 ms, 0.56 in two waves), unless all
-// pairs have the same number of events, one in every step: there the ranges
+// 0.6 / 0.95 sets: 0.308 -> 0.223, 0.353 -> 0.310, 0.376 -> 0.371 ms; FP64 1.17 ->
+// 0.99, 1.34 -> 1.27, 1.42 -> 1.44; level 5 FP32 0.181 -> 0.132, 0.216 -> 0.181, 0.228
+// -> 0.218; B1 level 10 0.89 -> 0.74, 1.04 -> 0.85, 1.49 -> 1.02).  For larger k lanes
+// that end early take the next pairs, which is worth more than the rest, unless
+// all pairs have the same number of events, one in every step: there the ranges
 // of FP32 launches are multiples of 32 up to k = 6 (level 4 at eps = 1e-3, k = 2:
-// 0.163 -> 0.121 ms, k = 6: 0.362 -> 0.341; FP64 launches lose, 0.52 -> 0.63 ms for
+// 0.158 -> 0.121 ms, k = 6: 0.347 -> 0.330; FP64 launches lose, 0.52 -> 0.63 ms for
 // 500 000 pairs of level 3).
 mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, const PairLaunch &P, int *grid,
                         unsigned long long *ppw)

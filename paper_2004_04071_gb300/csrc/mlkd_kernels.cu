@@ -39,8 +39,8 @@ template <typename Real> struct PhysState<Real, 1> { typedef HetPairState<Real> 
 // summed 32 at a time, so that neither path runs for only the few lanes that
 // fell idle together, and lanes wait less.  For coupled homogeneous pairs, with
 // a loop that holds nothing but the event (level 8 of the periodic problem,
-// 2^20 pairs: FP32 1.37 -> 1.21 ms, FP64 9.7 -> 8.9; 1000 pairs of level 10,
-// whose chains are all there is: 1.15 -> 0.87 ms, FP64 4.59 -> 4.42).  Uncoupled
+// 2^20 pairs: FP32 1.37 -> 1.20 ms, FP64 9.16 -> 8.54; 1000 pairs of level 10,
+// whose chains are all there is: 1.15 -> 0.86 ms, FP64 4.58 -> 4.30).  Uncoupled
 // pairs have so few events that the queues cost more than they save (5e6 paths
 // of level 0: FP32 0.18 ms without, 0.21 with them), and the heterogeneous
 // event is long enough (level 10 of B1: 2.39 and 2.43 ms).
