@@ -252,21 +252,40 @@ namespace {
 // of FP32 launches are multiples of 32 up to k = 6 (level 4 at eps = 1e-3, k = 2:
 // 0.158 -> 0.121 ms, k = 6: 0.347 -> 0.330; FP64 launches lose, 0.52 -> 0.63 ms for
 // 500 000 pairs of level 3).
-mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, const PairLaunch &P, int *grid,
+//
+// One pair per warp (32 of its events per step) instead of one per lane: for
+// coupled homogeneous FP64 pairs, while the chains of the lanes, not the work,
+// set the length of the launch.  A warp's work per pair goes with events + 32 (the
+// start and the last, partial step); the lines cross at 100 to 110 pairs per SM
+// times events / (events + 32) (measured at 2048, 512, 128, 64 and 32 events a
+// pair, one in every step: 16 000, 15 000, 13 500, 11 000, 8000 pairs on 152 SMs; with
+// longer flights later: level 8 at eps = 0.1 19 000).  1000 pairs of level 10 at
+// eps = 1e-3 (2048 events): 4.29 -> 0.39 ms; 100 of level 8 at eps = 0.1: 0.36 -> 0.04;
+// 4000: 0.39 -> 0.11.  Decisions and counts are the same, positions differ by
+// the order of their sums (rms error against extended precision 2e-16 to
+// 3.5e-16 on long pairs, 3e-16 to 1.5e-15 one pair per lane).  FP32 pairs keep the
+// lane form, whose rounding their results carry.
+constexpr double kWarpPairLeast = 32.0;
+constexpr double kWarpPairsPerSm = 100.0;
+
+mlkd_status choose_grid(int sm_count, int max_blocks, int mode, bool coupled, PairLaunch &P, int *grid,
                         unsigned long long *ppw)
 {
-    KernelInfo info;
-    if (pair_kernel_info(mode, coupled, P.nbins, &info, P.background) != cudaSuccess) return MLKD_ECUDA;
     const unsigned long long count = P.n_pairs;
+    // events expected per pair; fewer than half a step without a collision
+    const double events = -(double)P.n * std::expm1(-P.R * P.dt);
+    const bool fp64 = mode == kModeFP64 || mode == kModeFP64U24;
+    P.warp_pair = fp64 && coupled && P.background == 0 && events >= kWarpPairLeast &&
+                  (double)count * (events + 32.0) <= kWarpPairsPerSm * sm_count * events;
+    KernelInfo info;
+    if (pair_kernel_info(mode, coupled, P.nbins, &info, P.background, P.warp_pair != 0) != cudaSuccess) return MLKD_ECUDA;
     const long long wave = std::min<long long>((long long)sm_count * std::max(1, info.blocks_per_sm), max_blocks);
-    const unsigned long long per_block = 32ull * kWarpsPerBlock;
+    const unsigned long long per_block = (P.warp_pair ? 1ull : 32ull) * kWarpsPerBlock;
     const unsigned long long full = per_block * (unsigned long long)wave;
     unsigned long long g = std::min<unsigned long long>((count + per_block - 1) / per_block, (unsigned long long)wave);
     const unsigned long long k = count / full;
-    // events expected per pair; fewer than half a step without a collision
-    const double events = -(double)P.n * std::expm1(-P.R * P.dt);
-    const bool equal = mode != kModeFP64 && mode != kModeFP64U24 && (double)P.n * std::exp(-P.R * P.dt) < 0.5;
-    if (events >= 8.0 && (k == 1 || (equal && k >= 1 && k <= 6 && (double)(count % full) < 0.9 * (double)full))) {
+    const bool equal = !fp64 && (double)P.n * std::exp(-P.R * P.dt) < 0.5;
+    if (!P.warp_pair && events >= 8.0 && (k == 1 || (equal && k >= 1 && k <= 6 && (double)(count % full) < 0.9 * (double)full))) {
         const unsigned long long more = (count + k * per_block - 1) / (k * per_block);
         if (more <= (unsigned long long)max_blocks) g = more;
     }
@@ -331,7 +350,7 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.partial_rows = kMaxBlocks;
     P.arrived = ctx->arrived + (size_t)slot * kArrivals;
     if (accumulate) {
-        MLKD_CUDA(prefer_shared_memory(d.mode, level > 0, d.background));
+        MLKD_CUDA(prefer_shared_memory(d.mode, level > 0, P));
         P.acc = ctx->acc_stats + level;
         if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
     } else {

@@ -82,6 +82,7 @@ struct PairLaunch {
     uint32_t word2;            // level << 24 (pair_hi xor'ed in per pair)
     uint32_t request;
     int32_t fkind;             // F: 0 x^2, 1 (x mod 1)^2, 2 x
+    int32_t warp_pair;         // one pair per warp (FP64, coupled, homogeneous)
     int32_t background;        // 0 homogeneous, 1 B1, 2 B2 (heterogeneous kernel)
     double x0;                 // start of every path (init 2)
     double bg_b, bg_a_left, bg_a_right;   // R(x) = b (1 + a_l max(1-x,0) + a_r max(x-1,0))
@@ -113,14 +114,15 @@ struct KernelInfo {
 };
 
 // Kernel-variant occupancy (blocks per SM with kThreads threads).
-cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out, int background = 0);
+cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out, int background = 0,
+                             bool warp_pair = false);
 
 // Asks for the largest share of shared memory on the SMs that run the kernel
 // variant.  Variants that run at the same time (the levels of a round) then
 // want the same split of an SM and can share it: left to themselves the
 // uncoupled and the coupled kernel, which holds 16 to 21 KB a block, wait for
 // each other's SMs (an FP32 estimate of two levels 335 us, 296 with the same split).
-cudaError_t prefer_shared_memory(int mode, bool coupled, int background);
+cudaError_t prefer_shared_memory(int mode, bool coupled, const PairLaunch &p);
 
 // Launches the pair kernel on `grid` blocks.
 cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid,

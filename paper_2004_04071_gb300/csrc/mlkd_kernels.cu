@@ -15,6 +15,7 @@
 #include "mlkd_hetero.cuh"
 #include "mlkd_internal.h"
 #include "mlkd_pair.cuh"
+#include "mlkd_warp_pair.cuh"
 
 namespace mlkd {
 
@@ -176,7 +177,7 @@ __device__ __noinline__ void close_launch(const PairLaunch &P, double (*s_red)[k
     finish_launch(P, s_red[0]);
 }
 
-template <typename Real, int MODE, bool COUPLED, int PHYS>
+template <typename Real, int MODE, bool COUPLED, int PHYS, bool WARP = false>
 __global__ void __launch_bounds__(kThreads, (MinBlocks<Real, PHYS>::value))
 pair_kernel(const __grid_constant__ PairLaunch P)
 {
@@ -249,7 +250,7 @@ pair_kernel(const __grid_constant__ PairLaunch P)
     typename PhysState<Real, PHYS>::type st;
     st.fresh = true;
     // queues of started and finished pairs (see StartedPairs)
-    constexpr bool kQueues = COUPLED && PHYS == 0;
+    constexpr bool kQueues = COUPLED && PHYS == 0 && !WARP;
     // Sums in shared memory with queues (they change once per 32 pairs) and in
     // FP64, so that the event loop has the registers (FP32 coupled: 64, 8
     // blocks per SM).
@@ -291,7 +292,20 @@ pair_kernel(const __grid_constant__ PairLaunch P)
         }
     };
 
-    if constexpr (kQueues) {
+    if constexpr (WARP) {
+        // One pair per warp, 32 of its events per step (choose_grid has the
+        // rule); lane (pair mod 32) sums it.
+        for (pair = w_begin; pair < w_end; ++pair) {
+            bool none = pair_start<Real, CPL, RECIPE>(st, pair, L, P.keys, COUPLED);
+            if (P.init == 2) set_start(st, (Real)P.x0);
+            while (!none) none = warp_pair_step<Real, RECIPE>(st, L, P.keys, COUPLED, lane);
+            if (lane == (int)(pair & 31ull)) {
+                pair_drift<Real, CPL>(st, L, COUPLED);
+                account(st.xf, st.xc, st.k, st.evc);
+                record(pair, st.xf, st.xc, st.k, st.evc);
+            }
+        }
+    } else if constexpr (kQueues) {
     // warp-uniform: started pairs taken and held, the number of the first of
     // them, and the ring of finished pairs
     __shared__ StartedPairs<Real> s_started[kWarpsPerBlock];
@@ -685,7 +699,7 @@ namespace {
 typedef void (*PairKernelFn)(const PairLaunch);
 
 template <int PHYS>
-PairKernelFn pick_phys(int mode, bool coupled)
+PairKernelFn pick_lane(int mode, bool coupled)
 {
     switch (mode) {
     case kModeFP64:
@@ -702,26 +716,29 @@ PairKernelFn pick_phys(int mode, bool coupled)
     }
 }
 
-PairKernelFn pick(int mode, bool coupled, int background)
+PairKernelFn pick(int mode, bool coupled, int background, bool warp_pair)
 {
-    return background ? pick_phys<1>(mode, coupled) : pick_phys<0>(mode, coupled);
+    if (warp_pair)
+        return mode == kModeFP64 ? pair_kernel<double, kModeFP64, true, 0, true>
+                                 : pair_kernel<double, kModeFP64U24, true, 0, true>;
+    return background ? pick_lane<1>(mode, coupled) : pick_lane<0>(mode, coupled);
 }
 
 }  // namespace
 
-cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out, int background)
+cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out, int background, bool warp_pair)
 {
     int blocks = 0;
     const size_t smem = (size_t)3 * nbins * sizeof(unsigned int);
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &blocks, (const void *)pick(mode, coupled, background), kThreads, smem);
+        &blocks, (const void *)pick(mode, coupled, background, warp_pair), kThreads, smem);
     out->blocks_per_sm = blocks;
     return e;
 }
 
-cudaError_t prefer_shared_memory(int mode, bool coupled, int background)
+cudaError_t prefer_shared_memory(int mode, bool coupled, const PairLaunch &p)
 {
-    return cudaFuncSetAttribute((const void *)pick(mode, coupled, background),
+    return cudaFuncSetAttribute((const void *)pick(mode, coupled, p.background, p.warp_pair != 0),
                                 cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
 }
 
@@ -729,7 +746,7 @@ cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int 
                                cudaStream_t stream)
 {
     const size_t smem = (size_t)3 * p.nbins * sizeof(unsigned int);
-    pick(mode, coupled, p.background)<<<grid, kThreads, smem, stream>>>(p);
+    pick(mode, coupled, p.background, p.warp_pair != 0)<<<grid, kThreads, smem, stream>>>(p);
     return cudaGetLastError();
 }
 
