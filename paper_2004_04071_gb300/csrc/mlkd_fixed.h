@@ -212,7 +212,11 @@ MLKD_HD Pos pos_norm(uint64_t p, int e)                       // p 2^-e, p in [2
 MLKD_HD Pos operator*(const Pos &a, const Pos &b) { return pos_norm(mul64(a.m, b.m), a.e + b.e - 64); }
 // a times a fraction f 2^-64 of at least 1/2
 MLKD_HD Pos times(const Pos &a, uint64_t f) { return pos_norm(mul64(a.m, f), a.e); }
-MLKD_HD uint64_t bits_of(const Pos &a)                        // of the nearest double
+// The bits of the nearest double, for a.e <= 1084 (a number of at least 2^-1021;
+// e = 1086 with m = 2^63 gives 0).  The exponent field of a smaller one wraps:
+// squares and products of draws, which can be below that, go through
+// to_double_or_0.
+MLKD_HD uint64_t bits_of(const Pos &a)
 {
     return ((uint64_t)(1023 + 63 - 1 - a.e) << 52) + (a.m >> 11) + ((a.m >> 10) & 1u);
 }

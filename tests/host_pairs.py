@@ -1,0 +1,120 @@
+"""FP64 draws, coefficients and pairs of csrc/ compiled for the host: the
+same source as the kernels' (host_cuda/cuda_runtime.h stands in for CUDA), so
+that rare values can be fed to it without a GPU."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+SHIM = r"""
+#include "mlkd_pair.cuh"
+using namespace mlkd;
+// -ln u, nu and chi of the uniforms n1, n2, n3 (2^-B units), and the unit
+// coefficients of a phase of length s with that nu
+template <int B> static void draw1(const uint64_t *n, double s, double *out)
+{
+    const DrawFixed d = draw_fixed<B>(n[0], n[1], n[2], 1);
+    const Background<double>::Unit u = Background<double>::kd_unit<true>(fx::pos_of(s), d.nu * d.nu);
+    out[0] = d.nu_(), out[1] = d.chi_(), out[2] = fx::to_double(d.E), out[3] = u.D, out[4] = u.om, out[5] = u.beta;
+}
+extern "C" void draws(int B, const uint64_t *n, const double *s, int64_t count, double *out)
+{
+    init_draw_tables<double>();
+    for (int64_t i = 0; i < count; ++i)
+        B == 53 ? draw1<53>(n + 3 * i, s[i], out + 6 * i) : draw1<24>(n + 3 * i, s[i], out + 6 * i);
+}
+
+struct Least {
+    double least = 1.0;
+    void coarse(double, double E, double) { least = E < least ? E : least; }
+};
+struct Problem {
+    double R, mu, sigma, dt;
+    int32_t n, M, level;
+    uint32_t request;
+    uint64_t seed;
+};
+static LevelCtx<double> level_ctx(const Problem &p, PhiloxKeys &keys)
+{
+    LevelCtx<double> L;
+    L.bg.R = p.R, L.bg.invR = 1.0 / p.R, L.bg.mu = p.mu, L.bg.sigma = p.sigma;
+    L.bg.dt = p.dt, L.bg.Rdt = p.R * p.dt, L.bg.inv_Rdt = 1.0 / (p.R * p.dt);
+    L.bg.c = p.sigma / p.R, L.bg.c_lo = std::fma(-L.bg.c, p.R, p.sigma) / p.R;
+    L.n = p.n, L.M = p.M, L.init = 0, L.word2 = (uint32_t)p.level << 24, L.request = p.request;
+    L.divM.init(p.M);
+    for (int r = 0; r < 10; ++r) {
+        keys.k0[r] = (uint32_t)p.seed + (uint32_t)r * 0x9E3779B9u;
+        keys.k1[r] = (uint32_t)(p.seed >> 32) + (uint32_t)r * 0xBB67AE85u;
+    }
+    return L;
+}
+// positions at T and events of coupled pairs from the origin, and the
+// smallest coarse optical length E~ met
+template <int RECIPE>
+static double run(const Problem &p, uint64_t first, int64_t count, double *xf, double *xc, int32_t *kf, int32_t *kc)
+{
+    PhiloxKeys keys;
+    const LevelCtx<double> L = level_ctx(p, keys);
+    Least tr;
+    init_draw_tables<double>();
+    for (int64_t i = 0; i < count; ++i) {
+        PairState<double> st;
+        bool done = pair_start<double, 1, RECIPE>(st, first + (uint64_t)i, L, keys, true);
+        while (!done) done = pair_event<double, 1, RECIPE, Least>(st, L, keys, true, &tr);
+        pair_drift<double, 1>(st, L, true);
+        xf[i] = st.xf, xc[i] = st.xc, kf[i] = (int32_t)st.k, kc[i] = (int32_t)st.evc;
+    }
+    return tr.least;
+}
+extern "C" double pairs(int u24, const Problem *p, uint64_t first, int64_t count, double *xf, double *xc, int32_t *kf,
+                        int32_t *kc)
+{
+    return u24 ? run<1>(*p, first, count, xf, xc, kf, kc) : run<0>(*p, first, count, xf, xc, kf, kc);
+}
+"""
+
+
+class Problem(ctypes.Structure):
+    _fields_ = [("R", ctypes.c_double), ("mu", ctypes.c_double), ("sigma", ctypes.c_double), ("dt", ctypes.c_double),
+                ("n", ctypes.c_int32), ("M", ctypes.c_int32), ("level", ctypes.c_int32), ("request", ctypes.c_uint32),
+                ("seed", ctypes.c_uint64)]
+
+
+def build(folder):
+    src, so = os.path.join(folder, "shim.cpp"), os.path.join(folder, "shim.so")
+    with open(src, "w") as fh:
+        fh.write(SHIM)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", os.path.join(HERE, "host_cuda"),
+                    "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2004_04071_gb300", "csrc"), src,
+                    "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    lib.draws.restype = None
+    lib.pairs.restype = ctypes.c_double
+    return lib
+
+
+def ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def draws(lib, B, n, s):
+    """(nu, chi, E, D, om, beta) of the uniforms n[:, 3] 2^-B and phases of length s."""
+    n = np.ascontiguousarray(n, np.uint64)
+    s = np.ascontiguousarray(np.broadcast_to(np.asarray(s, np.float64), len(n)))
+    out = np.zeros((len(n), 6))
+    lib.draws(B, ptr(n), ptr(s), ctypes.c_int64(len(n)), ptr(out))
+    return out.T
+
+
+def pairs(lib, d, level, first, count, u24=False):
+    """xf, xc, kf, kc of coupled pairs of the free-space problem d, and the smallest E~."""
+    p = Problem(1.0 / (d["eps"] * d["eps"]), 0.0, 1.0 / d["eps"], d["dt0"] / d["M"] ** level,
+                int(round(d["T"] / d["dt0"])) * d["M"] ** level, d["M"], level, 0, d["seed"])
+    xf, xc = np.zeros(count), np.zeros(count)
+    kf, kc = np.zeros(count, np.int32), np.zeros(count, np.int32)
+    least = lib.pairs(int(u24), ctypes.byref(p), ctypes.c_uint64(first), ctypes.c_int64(count), ptr(xf), ptr(xc), ptr(kf), ptr(kc))
+    return xf, xc, kf, kc, least

@@ -1,0 +1,83 @@
+"""The FP64 draws, unit coefficients and pairs of the kernels, compiled for the
+host (host_pairs.py), at values that ordinary streams hardly ever meet,
+against extended precision and the oracle (no GPU).
+"""
+import numpy as np
+import pytest
+
+import host_pairs
+from helpers import fp64_close, oracle_problem
+
+LD = np.longdouble
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return host_pairs.build(str(tmp_path_factory.mktemp("host")))
+
+
+def unit_exact(s, nu):
+    """D, om and beta of a phase of length s with nu, in extended precision."""
+    s, nu = s.astype(LD), nu.astype(LD)
+    e, om = np.exp(-s), -np.expm1(-s)
+
+    def h(x):                                                          # e^-x + x - 1
+        small, t = np.minimum(x, 1), np.zeros_like(x)
+        for n in range(30, 1, -1):
+            t = (t + 1) * -small / (n + 1)
+        return np.where(x < 1, small * small / 2 * (1 + t), np.exp(-x) + x - 1)
+
+    # f = 2(e - 1) + s(e + 1) = sum_{n>=3} (-s)^n (2 - n)/n!
+    small, f = np.minimum(s, 1), np.zeros_like(s)
+    fact = np.cumprod(np.concatenate([[1], np.arange(1, 40)]).astype(LD))
+    for n in range(35, 2, -1):
+        f = f * -small + (2 - n) / fact[n]
+    f = np.where(s < 1, -f * small ** 3, s * (1 + e) - 2 * om)
+    g = np.where(s < 1, h(s) * om - f, 1 - 2 * s * e - e * e)          # g = h om - f
+    return np.sqrt(2 * f + nu * nu * g), om, np.sqrt(2 * h(h(s)))
+
+
+S = np.array([1e-300, 1e-9, 2.0**-64, 0.03, 0.5, np.nextafter(1.0, 0), 1.0, 1.5, 20.0, 43.99, 44.0, np.nextafter(64.0, 0), 64.0, 65.0,
+              1e3, 1e9, 1e100])
+
+
+@pytest.mark.parametrize("B", [53, 24])
+def test_coefficients_at_the_largest_uniform(lib, B):
+    """u1 = 1 gives nu = chi = 0 to FP64, at every phase and length: D is that
+    of nu = 0.  D: the terms are fixed-point numbers or two FP64 operations,
+    then a root (2 ulp); om: one rounding (1 ulp); beta for s >= 1: FP64
+    roundings of h (half an ulp each of h and om), magnified up to 2.5 times
+    in the root of 2 (e^-h + h - 1) (4 ulp)."""
+    phases = np.concatenate([np.arange(1, 17) << (B - 4), (np.arange(1, 17) << (B - 4)) - 3, [1, (1 << (B - 3)) + 1]])
+    n = np.array([[1 << B, p, 1 << B] for p in phases for _ in S], np.uint64)
+    s = np.tile(S, len(phases))
+    nu, chi, E, D, om, beta = host_pairs.draws(lib, B, n, s)
+    assert np.all(np.abs(nu) < 1e-150) and np.all(np.abs(chi) < 1e-150) and np.all(E == 0.0)
+    for got, exact, k in zip((D, om, beta), unit_exact(s, np.zeros(len(s))), (2, 1, 4)):
+        seen = exact >= 2.0**-1021                                     # smaller coefficients are 0
+        err = np.abs(got - exact)[seen] / np.spacing(got[seen])
+        assert np.all(err <= k), (float(np.max(err)), k, s[seen][np.argmax(err)])
+        assert np.all(got[~seen] == 0.0)
+
+
+@pytest.mark.parametrize("B", [53, 24])
+def test_coefficients_of_ordinary_draws(lib, B):
+    rng = np.random.default_rng(B)
+    n = rng.integers(1, 1 << B, (20000, 3)).astype(np.uint64)
+    s = np.concatenate([2.0 ** rng.uniform(-50, 0, 8000), rng.uniform(1, 64, 8000), 2.0 ** rng.uniform(6, 40, 4000)])
+    nu, _, _, D, om, beta = host_pairs.draws(lib, B, n, s)
+    for got, exact, k in zip((D, om, beta), unit_exact(s, nu), (2, 1, 4)):
+        assert np.max(np.abs(got - exact) / np.spacing(got)) <= k
+
+
+# pairs whose first coarse step is closed by an event with u1 = 1
+AT_ONE = [(41, 40879657), (41, 105628815), (1209, 2325), (1815, 9310), (80, 14745)]
+
+
+@pytest.mark.parametrize("seed,pair", AT_ONE)
+def test_pairs_that_draw_the_largest_uniform(lib, orc, seed, pair):
+    d = dict(eps=0.01, T=1.0, dt0=0.5, M=2, L=1, qoi=0, init=0, seed=seed)
+    xf_o, xc_o, kf_o, kc_o = orc.pairs(oracle_problem(orc, d, recipe=orc.RECIPE_24), 1, pair - 1, 3)
+    xf, xc, kf, kc, _ = host_pairs.pairs(lib, d, 1, pair - 1, 3, u24=True)
+    assert np.array_equal(kf, kf_o) and np.array_equal(kc, kc_o)
+    assert np.all(fp64_close(xf, xf_o)) and np.all(fp64_close(xc, xc_o))
