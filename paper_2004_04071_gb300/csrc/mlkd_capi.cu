@@ -35,12 +35,11 @@ Layout arena_layout()
         }
         return at;
     };
-    // one scratch slot (block partials, arrival counter) per level, so that the
+    // one scratch slot (block partials, arrival counters) per level, so that the
     // levels of a round can run at the same time
     L.partials = place((size_t)MLKD_MAX_LEVELS * kMaxBlocks * kPartialWords * sizeof(double));
     L.out = place(kOutHist + 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_stats = place(MLKD_MAX_LEVELS * sizeof(DevLevelStats));
-    L.tmp_hist = place(3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.acc_hist = place((size_t)MLKD_MAX_LEVELS * 3 * MLKD_MAX_BINS * sizeof(unsigned long long));
     L.arrived = place(MLKD_MAX_LEVELS * kArrivals * sizeof(unsigned long long));
     L.control = place(sizeof(DevControl));
@@ -348,17 +347,15 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.pairs_per_warp = ppw;
     P.partials = partials;
     P.partial_rows = kMaxBlocks;
-    P.arrived = ctx->arrived + (size_t)slot * kArrivals;
     if (accumulate) {
+        P.arrived = ctx->arrived + (size_t)slot * kArrivals;
         MLKD_CUDA(prefer_shared_memory(d.mode, level > 0, P));
         P.acc = ctx->acc_stats + level;
         if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
     } else {
+        P.arrived = (unsigned long long *)(ctx->out + kOutArrived);
         P.stats = (DevLevelStats *)ctx->out;
-        if (p->nbins > 0) {
-            P.hist = ctx->tmp_hist;
-            P.hist_out = (unsigned long long *)(ctx->out + kOutHist);
-        }
+        if (p->nbins > 0) P.hist = (unsigned long long *)(ctx->out + kOutHist);
     }
     P.dbg_xf = dxf;
     P.dbg_xc = dxc;
@@ -375,16 +372,13 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     return MLKD_OK;
 }
 
-// Zeroes the histogram scratch and the arrival counters, on the stream of the
-// first call and after a call that failed.  Every launch leaves the histogram
-// zero, and the counters below the next ticket.
-mlkd_status ensure_clean(mlkd_context *ctx, cudaStream_t s)
+// Zeroes what a call of one level counts in: its arrival counters and, behind
+// them, its histogram.  Every call does, so it reads nothing that an earlier
+// call, or the owner of the arena, left there.
+mlkd_status clear_counters(mlkd_context *ctx, int nbins, cudaStream_t s)
 {
-    if (!ctx->clean) {
-        MLKD_CUDA(cudaMemsetAsync(ctx->tmp_hist, 0, 3 * MLKD_MAX_BINS * sizeof(unsigned long long), s));
-        MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, MLKD_MAX_LEVELS * kArrivals * sizeof(unsigned long long), s));
-    }
-    ctx->clean = false;            // until the call has synchronised
+    MLKD_CUDA(cudaMemsetAsync(ctx->out + kOutArrived, 0,
+                              kOutHist - kOutArrived + 3 * (size_t)nbins * sizeof(unsigned long long), s));
     return MLKD_OK;
 }
 
@@ -483,9 +477,7 @@ mlkd_status mlkd_context_create(int device, void *arena, size_t arena_bytes, mlk
     c->partials = (double *)(c->arena + L.partials);
     c->out = c->arena + L.out;
     c->arrived = (unsigned long long *)(c->arena + L.arrived);
-    c->clean = false;
     c->acc_stats = (DevLevelStats *)(c->arena + L.acc_stats);
-    c->tmp_hist = (unsigned long long *)(c->arena + L.tmp_hist);
     c->acc_hist = (unsigned long long *)(c->arena + L.acc_hist);
     c->control = (DevControl *)(c->arena + L.control);
     if (kGuardBytes && (guards_write(c->arena, L.guard, L.n_guard, 0) != MLKD_OK ||
@@ -736,7 +728,7 @@ mlkd_status mlkd_run_level(mlkd_context *ctx, const mlkd_problem *problem, int l
         if (hist_out && problem->nbins > 0) std::memset(hist_out, 0, 3 * (size_t)problem->nbins * sizeof(uint64_t));
         return MLKD_OK;
     }
-    mlkd_status st = ensure_clean(ctx, s);
+    mlkd_status st = clear_counters(ctx, problem->nbins, s);
     if (st != MLKD_OK) return st;
     st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false, nullptr, nullptr, nullptr, nullptr);
     if (st != MLKD_OK) return st;
@@ -745,7 +737,6 @@ mlkd_status mlkd_run_level(mlkd_context *ctx, const mlkd_problem *problem, int l
     const size_t nh = hist_out ? 3 * (size_t)problem->nbins * sizeof(uint64_t) : 0;
     MLKD_CUDA(cudaMemcpyAsync(buf, ctx->out, nh ? kOutHist + nh : sizeof(DevLevelStats), cudaMemcpyDeviceToHost, s));
     MLKD_CUDA(cudaStreamSynchronize(s));
-    ctx->clean = true;
     DevLevelStats hs;
     std::memcpy(&hs, buf, sizeof(hs));
     to_host_stats(hs, out);
@@ -767,12 +758,11 @@ mlkd_status mlkd_debug_pairs(mlkd_context *ctx, const mlkd_problem *problem, int
     cudaStream_t s = (cudaStream_t)stream;
     MLKD_CUDA(cudaSetDevice(ctx->device));
     if (n_pairs == 0) return MLKD_OK;
-    mlkd_status st = ensure_clean(ctx, s);
+    mlkd_status st = clear_counters(ctx, problem->nbins, s);
     if (st != MLKD_OK) return st;
     st = enqueue_level(ctx, problem, d, level, first_pair, n_pairs, s, false, xf, xc, kf, kc);
     if (st != MLKD_OK) return st;
     MLKD_CUDA(cudaStreamSynchronize(s));
-    ctx->clean = true;
     return harvest_timing(ctx);
 }
 
@@ -833,10 +823,7 @@ static mlkd_status estimate_impl(mlkd_context *ctx, const mlkd_problem *problem,
     MLKD_CUDA(cudaMemsetAsync(ctx->acc_stats, 0, nl * sizeof(DevLevelStats), s));
     if (nb > 0)
         MLKD_CUDA(cudaMemsetAsync(ctx->acc_hist, 0, (size_t)nl * 3 * nb * sizeof(unsigned long long), s));
-    {
-        const mlkd_status cs = ensure_clean(ctx, s);
-        if (cs != MLKD_OK) return cs;
-    }
+    MLKD_CUDA(cudaMemsetAsync(ctx->arrived, 0, (size_t)nl * kArrivals * sizeof(unsigned long long), s));
     long long have[MLKD_MAX_LEVELS] = {0};
     const int density = problem->qoi == MLKD_QOI_DENSITY ? 1 : 0;
     DevControl ctl;
@@ -954,7 +941,6 @@ static mlkd_status estimate_impl(mlkd_context *ctx, const mlkd_problem *problem,
             for (int b = 0; b < nb; ++b) dens[b] /= d.h;
     }
     MLKD_CUDA(cudaStreamSynchronize(s));
-    ctx->clean = true;
     out->estimate = ctl.estimate;
     out->variance = ctl.variance;
     out->n_levels = nl;
@@ -1029,9 +1015,8 @@ constexpr size_t kNoAllocBytes = kNoAllocHistOffset + 3 * (size_t)MLKD_NOALLOC_M
 static_assert(kNoAllocBytes == (size_t)MLKD_NOALLOC_SCRATCH_BYTES, "scratch size mismatch");
 // the arrival counters share the level sums' slot (zero when the module is
 // loaded; a launch counts from its own ticket on)
-constexpr size_t kNoAllocArrivedOffset = kNoAllocStatsOffset + 128;
-static_assert(sizeof(DevLevelStats) <= 128 && kArrivals * sizeof(unsigned long long) <= 128,
-              "level sums or arrival counters exceed their scratch slot");
+constexpr size_t kNoAllocArrivedOffset = kNoAllocStatsOffset + kOutArrived;
+static_assert(kNoAllocHistOffset == kNoAllocStatsOffset + kOutHist, "a call's results lie as in an arena");
 
 }  // namespace
 

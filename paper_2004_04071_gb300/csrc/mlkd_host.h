@@ -31,7 +31,11 @@ constexpr size_t kAlign = 256;
 constexpr uint32_t kWeylA = 0x9E3779B9u;         // Philox key increments (SC'11)
 constexpr uint32_t kWeylB = 0xBB67AE85u;
 constexpr int kTimingRing = 64;
-constexpr size_t kOutHist = 256;                  // offset of a call's histogram behind its sums
+// A call of one level: its sums, at kOutArrived its arrival counters, and at
+// kOutHist its histogram (one clearing before it, one copy after it).
+constexpr size_t kOutArrived = 128, kOutHist = 256;
+static_assert(sizeof(DevLevelStats) <= kOutArrived && kArrivals * sizeof(unsigned long long) <= kOutHist - kOutArrived,
+              "level sums or arrival counters exceed their slot");
 
 // Canary bytes after each arena region in the debug build (MLKD_CHECKS):
 // written when the region is set up, compared after each synchronising call.
@@ -45,7 +49,7 @@ constexpr int kMaxGuards = 16;
 
 // Arena layout of the base workspace (offsets in bytes).
 struct Layout {
-    size_t partials, out, acc_stats, tmp_hist, acc_hist, arrived, control, total;
+    size_t partials, out, acc_stats, acc_hist, arrived, control, total;
     size_t guard[kMaxGuards];    // canary offsets (debug build)
     int n_guard;
 };
@@ -105,11 +109,10 @@ struct mlkd_context {
     size_t arena_bytes;
     mlkd::Layout L;
     double *partials;
-    char *out;                            // a call's sums and, kOutHist bytes on, its histogram
+    char *out;                            // sums, arrival counters and histogram of a call of one level
     mlkd::DevLevelStats *acc_stats;
-    unsigned long long *tmp_hist, *acc_hist;
-    unsigned long long *arrived;          // per scratch slot: arrival counters of the launch in flight
-    bool clean;                           // tmp_hist is zero (every launch leaves it so)
+    unsigned long long *acc_hist;
+    unsigned long long *arrived;          // per level of a round: arrival counters
     mlkd::DevControl *control;
     mlkd::BatchCache *batch;    // lazily created by the batched form
     mlkd::Server *server;       // running serving form, or null

@@ -96,7 +96,6 @@ struct PairLaunch {
     unsigned long long *arrived;       // [kArrivals], each ticket << kTicketShift | arrivals of that launch
     unsigned long long ticket;         // this launch, numbered upwards in a process
     DevLevelStats *stats, *acc;        // the launch's sums go to *stats and are added to *acc (or null)
-    unsigned long long *hist_out;      // hist is moved here and zeroed (or null: left in hist)
     double *dbg_xf, *dbg_xc;           // optional per-pair outputs
     int32_t *dbg_kf, *dbg_kc;
 };
