@@ -349,7 +349,6 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
     P.partial_rows = kMaxBlocks;
     if (accumulate) {
         P.arrived = ctx->arrived + (size_t)slot * kArrivals;
-        MLKD_CUDA(prefer_shared_memory(d.mode, level > 0, P));
         P.acc = ctx->acc_stats + level;
         if (p->nbins > 0) P.hist = ctx->acc_hist + (size_t)level * 3 * p->nbins;
     } else {
@@ -367,7 +366,7 @@ mlkd_status enqueue_level(mlkd_context *ctx, const mlkd_problem *p, const Derive
         if (st2 != MLKD_OK) return st2;
     }
     if (timed) MLKD_CUDA(cudaEventRecord(ctx->ev_start[ctx->pending], stream));
-    MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, stream));
+    MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, stream, accumulate));
     if (timed) MLKD_CUDA(cudaEventRecord(ctx->ev_stop[ctx->pending++], stream));
     return MLKD_OK;
 }
@@ -1119,7 +1118,7 @@ extern "C" mlkd_status mlkd_run_level_noalloc(const mlkd_problem *problem, int l
     P.arrived = (unsigned long long *)(scratch + kNoAllocArrivedOffset);
     if (problem->nbins > 0)   // counters keep the previous call's values
         MLKD_CUDA(cudaMemsetAsync(P.hist, 0, 3 * (size_t)problem->nbins * sizeof(unsigned long long), s));
-    MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, s));
+    MLKD_CUDA(launch_pair_kernel(d.mode, level > 0, P, grid, s, false));
     // sums and histogram lie one behind the other: one copy
     unsigned char buf[256 + 3 * MLKD_NOALLOC_MAX_BINS * sizeof(uint64_t)];
     const size_t nh = hist_out ? 3 * (size_t)problem->nbins * sizeof(uint64_t) : 0;

@@ -116,16 +116,15 @@ struct KernelInfo {
 cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out, int background = 0,
                              bool warp_pair = false);
 
-// Asks for the largest share of shared memory on the SMs that run the kernel
-// variant.  Variants that run at the same time (the levels of a round) then
-// want the same split of an SM and can share it: left to themselves the
-// uncoupled and the coupled kernel, which holds 16 to 21 KB a block, wait for
-// each other's SMs (an FP32 estimate of two levels 335 us, 296 with the same split).
-cudaError_t prefer_shared_memory(int mode, bool coupled, const PairLaunch &p);
-
-// Launches the pair kernel on `grid` blocks.
-cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid,
-                               cudaStream_t stream);
+// Launches the pair kernel on `grid` blocks.  max_shared asks for the largest
+// share of shared memory on the SMs that run this launch (an attribute of the
+// launch, not of the kernel: later launches are as before).  Kernel variants
+// that run at the same time (the levels of a round) then want the same split
+// of an SM and can share it: left to themselves the uncoupled and the coupled
+// kernel, which holds 16 to 21 KB a block, wait for each other's SMs (an FP32
+// estimate of two levels 335 us, 296 with the same split).
+cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid, cudaStream_t stream,
+                               bool max_shared);
 
 // Output of the on-device sample-count controller (eqs. Nopt1/Noptj).
 struct DevControl {

@@ -729,18 +729,22 @@ cudaError_t pair_kernel_info(int mode, bool coupled, int nbins, KernelInfo *out,
     return e;
 }
 
-cudaError_t prefer_shared_memory(int mode, bool coupled, const PairLaunch &p)
+cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid, cudaStream_t stream,
+                               bool max_shared)
 {
-    return cudaFuncSetAttribute((const void *)pick(mode, coupled, p.background, p.warp_pair != 0),
-                                cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-}
-
-cudaError_t launch_pair_kernel(int mode, bool coupled, const PairLaunch &p, int grid,
-                               cudaStream_t stream)
-{
-    const size_t smem = (size_t)3 * p.nbins * sizeof(unsigned int);
-    pick(mode, coupled, p.background, p.warp_pair != 0)<<<grid, kThreads, smem, stream>>>(p);
-    return cudaGetLastError();
+    cudaLaunchAttribute split;
+    split.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    split.val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = (size_t)3 * p.nbins * sizeof(unsigned int);
+    cfg.stream = stream;
+    cfg.attrs = &split;
+    cfg.numAttrs = max_shared ? 1u : 0u;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(mode, coupled, p.background, p.warp_pair != 0), p);
+    if (e != cudaSuccess) cudaGetLastError();     // returned here, not left for the caller's next check
+    return e;
 }
 
 cudaError_t launch_controller(const DevLevelStats *acc, const unsigned long long *hist_acc,
