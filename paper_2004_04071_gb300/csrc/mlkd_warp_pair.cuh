@@ -64,7 +64,8 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
         vp = st.vf;
     }
     // step count floor(q) + 1, its prefix sum saturated at n + 1 (only
-    // events with an index below n are ever taken)
+    // events with an index below n are ever taken); two such sums reach
+    // 2^31 + 2, so they are added unsigned
     const int n = L.n;
     const Real qpc = A::min_(qp, (Real)n);
     const int sq = (int)qpc;
@@ -74,17 +75,18 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
     // below take that shortcut when it holds for the whole step; their
     // results are the same values either way.
     const bool one_step = __all_sync(kFullMask, qp < Real(1) && qn < Real(1));
-    int ia = sq + 1;                                           // inclusive prefix -> index after
+    const unsigned most = (unsigned)n + 1u;
+    unsigned sum = (unsigned)sq + 1u;                          // inclusive prefix
     if (one_step) {
-        ia = lane + 1;
+        sum = (unsigned)lane + 1u;
     } else {
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const int up = __shfl_up_sync(kFullMask, ia, off);
-            if (lane >= off) ia = min(ia + up, n + 1);
+            const unsigned up = __shfl_up_sync(kFullMask, sum, off);
+            if (lane >= off) sum = min(sum + up, most);
         }
     }
-    ia = min(st.i_f + ia, n + 1);
+    const int ia = (int)min((unsigned)st.i_f + sum, most);     // index after this event
     const int ib = ia - (sq + 1);                              // index before this event
     const bool valid = qp < (Real)(n - ib);                    // previous collision before T
     const unsigned vmask = __ballot_sync(kFullMask, valid);

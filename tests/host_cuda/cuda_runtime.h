@@ -1,9 +1,11 @@
-// The names of CUDA that csrc/mlkd_device.cuh and mlkd_pair.cuh use, for one
-// host thread: lets a CPU test call the functions of the FP64 pairs.
+// The names of CUDA that the pairs of csrc/ use, on the host: lets a CPU test
+// call the functions of the FP64 pairs.  A warp is 32 threads that meet in
+// every shuffle and vote.
 #pragma once
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <pthread.h>
 
 #define __device__
 #define __host__
@@ -23,7 +25,38 @@ struct uint4 {
 static inline uint4 make_uint4(uint32_t x, uint32_t y, uint32_t z, uint32_t w) { return uint4{x, y, z, w}; }
 static const struct { unsigned x; } threadIdx = {0}, blockDim = {1};
 static inline void __syncthreads() {}
-template <typename T> static inline T __shfl_down_sync(unsigned, T v, int) { return v; }
+
+static thread_local int host_lane = 0;
+static pthread_barrier_t host_warp;             // of 32
+static uint64_t host_words[32];
+template <typename T, typename F> static inline T host_exchange(T v, F from)
+{
+    uint64_t w = 0;
+    memcpy(&w, &v, sizeof v);
+    host_words[host_lane] = w;
+    pthread_barrier_wait(&host_warp);
+    const int l = from(host_lane);
+    w = host_words[l >= 0 && l < 32 ? l : host_lane];
+    pthread_barrier_wait(&host_warp);
+    memcpy(&v, &w, sizeof v);
+    return v;
+}
+template <typename T> static inline T __shfl_sync(unsigned, T v, int l) { return host_exchange(v, [=](int) { return l & 31; }); }
+template <typename T> static inline T __shfl_up_sync(unsigned, T v, int d) { return host_exchange(v, [=](int l) { return l - d; }); }
+template <typename T> static inline T __shfl_down_sync(unsigned, T v, int d) { return host_exchange(v, [=](int l) { return l + d; }); }
+template <typename T> static inline T __shfl_xor_sync(unsigned, T v, int d) { return host_exchange(v, [=](int l) { return l ^ d; }); }
+static inline unsigned __ballot_sync(unsigned, bool p)
+{
+    host_words[host_lane] = p;
+    pthread_barrier_wait(&host_warp);
+    unsigned m = 0;
+    for (int l = 0; l < 32; ++l) m |= (unsigned)host_words[l] << l;
+    pthread_barrier_wait(&host_warp);
+    return m;
+}
+static inline bool __all_sync(unsigned m, bool p) { return __ballot_sync(m, p) == 0xffffffffu; }
+static inline int __popc(unsigned x) { return __builtin_popcount(x); }
+static inline int __clz(int x) { return x ? __builtin_clz((unsigned)x) : 32; }
 
 template <typename A, typename B> static inline A host_bits(B b)
 {

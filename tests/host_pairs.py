@@ -11,7 +11,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 
 SHIM = r"""
-#include "mlkd_pair.cuh"
+#include <thread>
+#include <vector>
+#include "mlkd_warp_pair.cuh"
 using namespace mlkd;
 // -ln u, nu and chi of the uniforms n1, n2, n3 (2^-B units), and the unit
 // coefficients of a phase of length s with that nu
@@ -75,6 +77,40 @@ extern "C" double pairs(int u24, const Problem *p, uint64_t first, int64_t count
 {
     return u24 ? run<1>(*p, first, count, xf, xc, kf, kc) : run<0>(*p, first, count, xf, xc, kf, kc);
 }
+// the same pairs, each by a warp; a pair that takes more than `most` steps is
+// left there with kf = -1
+template <int RECIPE>
+static void run_warps(const Problem &p, uint64_t first, int64_t count, int most, double *xf, double *xc, int32_t *kf, int32_t *kc)
+{
+    PhiloxKeys keys;
+    const LevelCtx<double> L = level_ctx(p, keys);
+    init_draw_tables<double>();
+    pthread_barrier_init(&host_warp, nullptr, 32);
+    std::vector<std::thread> lanes;
+    for (int lane = 0; lane < 32; ++lane)
+        lanes.emplace_back([&, lane] {
+            host_lane = lane;
+            for (int64_t i = 0; i < count; ++i) {
+                PairState<double> st;
+                bool done = pair_start<double, 1, RECIPE>(st, first + (uint64_t)i, L, keys, true);
+                int steps = 0;
+                while (!done && steps < most) {
+                    done = warp_pair_step<double, RECIPE>(st, L, keys, true, lane);
+                    ++steps;
+                }
+                pair_drift<double, 1>(st, L, true);
+                if (lane == 0) xf[i] = st.xf, xc[i] = st.xc, kf[i] = done ? (int32_t)st.k : -1, kc[i] = (int32_t)st.evc;
+            }
+        });
+    for (auto &t : lanes) t.join();
+    pthread_barrier_destroy(&host_warp);
+}
+extern "C" void warp_pairs(int u24, const Problem *p, uint64_t first, int64_t count, int most, double *xf, double *xc,
+                           int32_t *kf, int32_t *kc)
+{
+    if (u24) run_warps<1>(*p, first, count, most, xf, xc, kf, kc);
+    else run_warps<0>(*p, first, count, most, xf, xc, kf, kc);
+}
 """
 
 
@@ -88,11 +124,11 @@ def build(folder):
     src, so = os.path.join(folder, "shim.cpp"), os.path.join(folder, "shim.so")
     with open(src, "w") as fh:
         fh.write(SHIM)
-    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", os.path.join(HERE, "host_cuda"),
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-fwrapv", "-pthread", "-shared", "-fPIC", "-I", os.path.join(HERE, "host_cuda"),
                     "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2004_04071_gb300", "csrc"), src,
                     "-o", so], check=True)
     lib = ctypes.CDLL(so)
-    lib.draws.restype = None
+    lib.draws.restype = lib.warp_pairs.restype = None
     lib.pairs.restype = ctypes.c_double
     return lib
 
@@ -110,11 +146,19 @@ def draws(lib, B, n, s):
     return out.T
 
 
-def pairs(lib, d, level, first, count, u24=False):
-    """xf, xc, kf, kc of coupled pairs of the free-space problem d, and the smallest E~."""
-    p = Problem(1.0 / (d["eps"] * d["eps"]), 0.0, 1.0 / d["eps"], d["dt0"] / d["M"] ** level,
-                int(round(d["T"] / d["dt0"])) * d["M"] ** level, d["M"], level, 0, d["seed"])
+def problem(d, level):
+    return Problem(1.0 / (d["eps"] * d["eps"]), 0.0, 1.0 / d["eps"], d["dt0"] / d["M"] ** level,
+                   int(round(d["T"] / d["dt0"])) * d["M"] ** level, d["M"], level, 0, d["seed"])
+
+
+def pairs(lib, d, level, first, count, u24=False, warp=0):
+    """xf, xc, kf, kc of coupled pairs of the free-space problem d, and the
+    smallest E~; warp: one pair per warp, that many steps at most."""
     xf, xc = np.zeros(count), np.zeros(count)
     kf, kc = np.zeros(count, np.int32), np.zeros(count, np.int32)
-    least = lib.pairs(int(u24), ctypes.byref(p), ctypes.c_uint64(first), ctypes.c_int64(count), ptr(xf), ptr(xc), ptr(kf), ptr(kc))
+    at = (ctypes.byref(problem(d, level)), ctypes.c_uint64(first), ctypes.c_int64(count))
+    if warp:
+        lib.warp_pairs(int(u24), *at, warp, ptr(xf), ptr(xc), ptr(kf), ptr(kc))
+        return xf, xc, kf, kc, None
+    least = lib.pairs(int(u24), *at, ptr(xf), ptr(xc), ptr(kf), ptr(kc))
     return xf, xc, kf, kc, least

@@ -81,3 +81,17 @@ def test_pairs_that_draw_the_largest_uniform(lib, orc, seed, pair):
     xf, xc, kf, kc, _ = host_pairs.pairs(lib, d, 1, pair - 1, 3, u24=True)
     assert np.array_equal(kf, kf_o) and np.array_equal(kc, kc_o)
     assert np.all(fp64_close(xf, xf_o)) and np.all(fp64_close(xc, xc_o))
+
+
+@pytest.mark.parametrize("eps,level", [(0.7, 15), (0.1, 15), (0.7, 13), (0.05, 3)])
+def test_warp_form_with_the_most_steps(lib, eps, level):
+    """One pair per warp at 2^30 fine steps, the most there are, and at fewer:
+    the events of the one-lane form, and its positions to the order of their
+    sums (some 100 numbers of order 1, rounded at 2^-53)."""
+    d = dict(eps=eps, T=1.0, dt0=1.0, M=4, seed=41)
+    lane = host_pairs.pairs(lib, d, level, 0, 24)
+    warp = host_pairs.pairs(lib, d, level, 0, 24, warp=400)
+    for a, b in zip(warp[2:4], lane[2:4]):
+        assert np.array_equal(a, b)
+    for a, b in zip(warp[:2], lane[:2]):
+        assert np.all(fp64_close(a, b, 1e-13))
