@@ -27,11 +27,11 @@ struct NoTrace {};
 // FP64 state is dimensionless: with velocities mu + sigma nu, the position
 // is x = x_0 + mu t + (sigma/R) y, a kinetic phase of optical length E moves y by
 // nu E, and no coefficient of the background is left in the KD step but R dt.
-// xf, xc hold y and vf, vc hold nu.  One pair per lane keeps a flight as its
-// optical length and its split into whole steps and the rest of the
-// collision's step; one pair per warp keeps it as qf, qc.
-// FP32 keeps its floor beside qf.
+// xf, xc hold y and vf, vc hold nu.  A flight is kept as its optical length and
+// its split into whole steps and the rest of the collision's step.
+// FP32 keeps the flight in fine steps and its floor.
 template <typename Real> struct FlightState {
+    Real qf, qc;
     int whole_f;                // floor(qf)
 };
 template <> struct FlightState<double> {
@@ -42,8 +42,8 @@ template <> struct FlightState<double> {
 };
 
 template <typename Real> struct PairState : FlightState<Real> {
-    Real xf, vf, qf;            // fine path: position, velocity, flight (fine units)
-    Real xc, vc, qc;            // coarse path
+    Real xf, vf;                // fine path: position, velocity
+    Real xc, vc;                // coarse path
     Real num, den, chi_first;   // streamed eq. chi-update of the open coarse window
     int i_f, ic, Ec;            // fine-step index of each path's phase start; coarse step end
     uint32_t k, evc;            // fine events (= Philox block of the next draw - 1), coarse events
@@ -139,7 +139,6 @@ __device__ __forceinline__ bool pair_init(PairState<Real> &st, unsigned long lon
     const Real qf = first_flight(L, q0);
     set_start(st, x0);
     st.vf = v0;
-    st.qf = qf;
     st.i_f = 0;
     st.k = 0;
     st.evc = 0;
@@ -151,11 +150,11 @@ __device__ __forceinline__ bool pair_init(PairState<Real> &st, unsigned long lon
         st.whole_f = st.whole_c = fl.whole;
         st.left_f = st.left_c = fl.left;
     } else {
+        st.qf = st.qc = qf;
         whole = st.whole_f = __float2int_rz(qf);
     }
     if (coupled) {
         st.vc = v0;
-        st.qc = qf;
         st.ic = 0;
         st.num = Real(0);
         st.den = Real(0);

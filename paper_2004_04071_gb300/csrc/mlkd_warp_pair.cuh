@@ -50,31 +50,63 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
 {
     typedef Arith<Real> A;
     const Background<Real> &bg = L.bg;
-    const Draw<Real> d = draw_r<Real, RECIPE>(st.k + 1u + (uint32_t)lane, st.pair_lo, st.word2,
-                                              L.request, keys);
-    const Real qn = d.E * bg.inv_Rdt;                          // flight after this event
-    // FP64 state is dimensionless: v1 holds nu (see PairState)
+    const int n = L.n;
+    // FP64 state is dimensionless (see PairState): dv and v1 hold nu, and a
+    // flight is its optical length and its split into whole steps and a rest
     constexpr bool kUnit = std::is_same<Real, double>::value;
-    const Real dv = kUnit ? d.nu : bg.sigma * d.nu;            // v_{k+1} - mu
-    const Real v1 = kUnit ? d.nu : bg.mu + dv;
-    Real qp = __shfl_up_sync(kFullMask, qn, 1);                // flight before this event
+    Real nu, chi, dv, v1;
+    Real qn = Real(0), qp = Real(0);                           // FP32: flight after this event, and before it
+    Real En = Real(0), Ep = Real(0);                           // FP64: the same as optical length
+    uint64_t left_n = 0, left_p = 0;                           // and the rest of the collision's step
+    int wn, wp;                                                // their whole steps (FP32: at most n)
+    fx::Pos nu2;
+    if constexpr (kUnit) {
+        const DrawFixed d = draw_fixed_r<RECIPE>(st.k + 1u + (uint32_t)lane, st.pair_lo, st.word2, L.request, keys);
+        nu = dv = v1 = d.nu_();
+        chi = d.chi_();
+        nu2 = d.nu * d.nu;
+        En = fx::to_double(d.E);
+        const fx::Flight fl = fx::split_flight(d.E * fx::pos_of(bg.inv_Rdt));
+        wn = fl.whole;
+        left_n = fl.left;
+        wp = __shfl_up_sync(kFullMask, wn, 1);
+        left_p = __shfl_up_sync(kFullMask, left_n, 1);
+        Ep = __shfl_up_sync(kFullMask, En, 1);
+    } else {
+        const Draw<Real> d = draw_r<Real, RECIPE>(st.k + 1u + (uint32_t)lane, st.pair_lo, st.word2,
+                                                  L.request, keys);
+        nu = d.nu;
+        chi = d.chi;
+        dv = bg.sigma * nu;                                    // v_{k+1} - mu
+        v1 = bg.mu + dv;
+        qn = d.E * bg.inv_Rdt;
+        qp = __shfl_up_sync(kFullMask, qn, 1);
+    }
     Real vp = __shfl_up_sync(kFullMask, v1, 1);
     if (lane == 0) {
-        qp = st.qf;
         vp = st.vf;
+        if constexpr (kUnit) {
+            wp = st.whole_f;
+            left_p = st.left_f;
+            Ep = st.of;
+        } else {
+            qp = st.qf;
+        }
+    }
+    if constexpr (!kUnit) {
+        wn = (int)A::min_(qn, (Real)n);
+        wp = (int)A::min_(qp, (Real)n);
     }
     // step count floor(q) + 1, its prefix sum saturated at n + 1 (only
     // events with an index below n are ever taken); two such sums reach
     // 2^31 + 2, so they are added unsigned
-    const int n = L.n;
-    const Real qpc = A::min_(qp, (Real)n);
-    const int sq = (int)qpc;
+    const int sq = min(wp, n);
     // In the diffusive regime every flight is shorter than a fine step
     // (R dt >> 1): each event then advances one step, the prefix sum is the
     // lane index, and a coarse window holds at most M events.  The scans
     // below take that shortcut when it holds for the whole step; their
     // results are the same values either way.
-    const bool one_step = __all_sync(kFullMask, qp < Real(1) && qn < Real(1));
+    const bool one_step = __all_sync(kFullMask, wp < 1 && wn < 1);
     const unsigned most = (unsigned)n + 1u;
     unsigned sum = (unsigned)sq + 1u;                          // inclusive prefix
     if (one_step) {
@@ -88,38 +120,37 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
     }
     const int ia = (int)min((unsigned)st.i_f + sum, most);     // index after this event
     const int ib = ia - (sq + 1);                              // index before this event
-    const bool valid = qp < (Real)(n - ib);                    // previous collision before T
+    const bool valid = wp < n - ib;                            // previous collision before T
     const unsigned vmask = __ballot_sync(kFullMask, valid);
     const int nvalid = __popc(vmask);                          // a prefix of the lanes
     const int last = nvalid - 1;
 
     Real a, dd, hs, om, dx = Real(0), bh = Real(0);
     if constexpr (kUnit) {
-        const double s = bg.Rdt * ((double)(sq + 1) - qp);
-        const Background<double>::Unit f = Background<double>::kd_unit<true>(fx::pos_of(s), fx::pos_of(dv * dv));
+        const Background<double>::Unit f =
+            Background<double>::kd_unit<true>(fx::pos_of(bg.Rdt) * fx::steps_left(0, left_p), nu2);
         om = f.om;
         bh = f.beta;
-        if (valid) dx = fma(f.D, d.chi, fma(dv, om, vp * (qp * bg.Rdt)));
+        if (valid) dx = fma(vp, Ep, fma(f.D, chi, dv * om));
     } else {
         const Real theta = bg.dt * ((Real)(sq + 1) - qp);      // eq. diffusive-time
         bg.kd_coeffs(theta, dv, a, dd, hs, om);
-        dx = valid ? vp * (qp * bg.dt) + (a + dd * d.chi) : Real(0);   // eq. position-update
+        dx = valid ? vp * (qp * bg.dt) + (a + dd * chi) : Real(0);   // eq. position-update
     }
     st.xf = st.xf + warp_sum(dx);
 
     bool done;
     {
-        const Real ql = __shfl_sync(kFullMask, qn, last);
+        const int wl = __shfl_sync(kFullMask, wn, last);
         const Real vl = __shfl_sync(kFullMask, v1, last);
         const int il = __shfl_sync(kFullMask, ia, last);
-        done = !(ql < (Real)(n - il));
+        done = !(wl < n - il);
         if (coupled) {
             // ---- coarse window: triggers, window sums, coarse steps ----
-            const int qnc = (int)A::min_(qn, (Real)n);
             // floor of the collision after, clamped at n: any collision at or
             // after T lies past the coarse step of the one before it (n is a
             // multiple of M), so the clamp changes no trigger
-            const int cfl = ia + min(qnc, n - min(ia, n));
+            const int cfl = ia + min(min(wn, n), n - min(ia, n));
             const int Kn = L.divM(cfl);
             int Kp = __shfl_up_sync(kFullMask, Kn, 1);
             if (lane == 0) Kp = L.divM(st.Ec) - 1;             // coarse step of the carried collision
@@ -128,11 +159,11 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             Real bh2;
             if constexpr (kUnit) bh2 = bh * bh;
             else bh = bg.beta_hat(hs, bh2);
-            Real cn = valid ? bh * d.chi : Real(0);
+            Real cn = valid ? bh * chi : Real(0);
             Real cd = valid ? bh2 : Real(0);
             if (valid && !trig) {
-                const Real ah = qn * bg.Rdt + om;              // R tau' = R tau + R zeta
-                cn += ah * d.nu;
+                const Real ah = (kUnit ? En : qn * bg.Rdt) + om;   // R tau' = R tau + R zeta
+                cn += ah * nu;
                 cd += ah * ah;
             }
             // segmented inclusive scan; a window starts after each trigger.
@@ -160,23 +191,42 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             const int src = p >= 0 ? p : 0;
             const int ecp = L.M * (Kp + 1);                    // coarse step end in force
             // post-trigger coarse state of each lane (used from its trigger lanes)
-            const Real qc_post = qn - (Real)(ecp - ia);
+            const int to_end = ecp - ia;
+            int wc_post = 0;
+            Real qc_post;                                      // FP64: optical length
+            if constexpr (kUnit) {
+                wc_post = wn - to_end;
+                qc_post = to_end > 0 ? fma(-fx::from_u32((uint32_t)to_end), bg.Rdt, En) : En;
+            } else {
+                qc_post = qn - (Real)to_end;
+            }
             const int ic_from = __shfl_sync(kFullMask, ecp, src);      // ic after trigger p
             const Real qc_from = __shfl_sync(kFullMask, qc_post, src);
             const Real vc_from = __shfl_sync(kFullMask, v1, src);
             const int ic_pre = p >= 0 ? ic_from : st.ic;
-            const Real qc_pre = p >= 0 ? qc_from : st.qc;
             const Real vc_pre = p >= 0 ? vc_from : st.vc;
-            const Real chi_head = __shfl_sync(kFullMask, d.chi, p + 1 < 32 ? p + 1 : 31);
+            Real qc_pre;
+            int wc_pre = 0;
+            uint64_t left_pre = 0;
+            if constexpr (kUnit) {
+                const int wc_from = __shfl_sync(kFullMask, wc_post, src);
+                const uint64_t left_from = __shfl_sync(kFullMask, left_n, src);
+                qc_pre = p >= 0 ? qc_from : st.oc;
+                wc_pre = p >= 0 ? wc_from : st.whole_c;
+                left_pre = p >= 0 ? left_from : st.left_c;
+            } else {
+                qc_pre = p >= 0 ? qc_from : st.qc;
+            }
+            const Real chi_head = __shfl_sync(kFullMask, chi, p + 1 < 32 ? p + 1 : 31);
             const Real chi_first = (p < 0 && !st.fresh) ? st.chi_first : chi_head;
             Real dxc = Real(0);
             if (trig) {
                 Real ac, dc, omc;
                 const Real chit = cd > Real(0) ? cn * A::rsqrt_(cd) : chi_first;
                 if constexpr (kUnit) {
-                    const double sc = bg.Rdt * ((double)(ecp - ic_pre) - qc_pre);
-                    const Background<double>::Unit c = Background<double>::kd_unit<false>(fx::pos_of(sc), fx::pos_of(dv * dv));
-                    dxc = fma(c.D, chit, fma(dv, c.om, vc_pre * (qc_pre * bg.Rdt)));
+                    const fx::Pos sc = fx::pos_of(bg.Rdt) * fx::steps_left(ecp - ic_pre - wc_pre - 1, left_pre);
+                    const Background<double>::Unit c = Background<double>::kd_unit<false>(sc, nu2);
+                    dxc = fma(vc_pre, qc_pre, fma(c.D, chit, dv * c.om));
                 } else {
                     const Real thc = bg.dt * ((Real)(ecp - ic_pre) - qc_pre);
                     Real hsc;
@@ -192,9 +242,16 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
                 const int ic_t = __shfl_sync(kFullMask, ecp, t);
                 const Real qc_t = __shfl_sync(kFullMask, qc_post, t);
                 st.ic = ic_t;
-                st.qc = qc_t;
                 st.vc = __shfl_sync(kFullMask, v1, t);
-                if (qc_t < (Real)(n - ic_t)) st.Ec = next_coarse_end(L, ic_t, (int)qc_t);
+                if constexpr (kUnit) {
+                    st.oc = qc_t;
+                    st.whole_c = __shfl_sync(kFullMask, wc_post, t);
+                    st.left_c = __shfl_sync(kFullMask, left_n, t);
+                    if (st.whole_c < n - ic_t) st.Ec = next_coarse_end(L, ic_t, st.whole_c);
+                } else {
+                    st.qc = qc_t;
+                    if (qc_t < (Real)(n - ic_t)) st.Ec = next_coarse_end(L, ic_t, (int)qc_t);
+                }
             }
             const bool trig_last = (tmask >> last) & 1u;
             const Real num_l = __shfl_sync(kFullMask, cn, last);
@@ -213,8 +270,14 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
         }
         st.k += (uint32_t)nvalid;
         st.i_f = il;
-        st.qf = ql;
         st.vf = vl;
+        if constexpr (kUnit) {
+            st.whole_f = wl;
+            st.left_f = __shfl_sync(kFullMask, left_n, last);
+            st.of = __shfl_sync(kFullMask, En, last);
+        } else {
+            st.qf = __shfl_sync(kFullMask, qn, last);
+        }
     }
     return done;
 }

@@ -162,3 +162,12 @@ def pairs(lib, d, level, first, count, u24=False, warp=0):
         return xf, xc, kf, kc, None
     least = lib.pairs(int(u24), *at, ptr(xf), ptr(xc), ptr(kf), ptr(kc))
     return xf, xc, kf, kc, least
+
+
+# (eps, pair, 24-bit stream) of level 6 of BOUNDARY: E / (R dt) of one of the
+# pair's first events is below a whole number by less than FP64 resolves
+BOUNDARY = dict(T=1.0, dt0=0.5, M=2, L=6, seed=59, qoi=0, init=0)
+AT_BOUNDARY = [(float.fromhex(e), pair, u24) for e, pair, u24 in (
+    ("0x1.5ab3fced1e871p-4", 1, False), ("0x1.ea4fec05af416p-4", 1, False), ("0x1.0608ee7b3f7a3p-3", 5, False),
+    ("0x1.c784eeb88ed90p-4", 7, False), ("0x1.5f18e07268fccp-4", 9, False), ("0x1.e40e71800ea5ap-4", 2, True),
+    ("0x1.cd1257f72e48cp-4", 4, True), ("0x1.b79b2aeed81c9p-4", 10, True), ("0x1.cc76e56447539p-4", 17, True))]

@@ -95,3 +95,14 @@ def test_warp_form_with_the_most_steps(lib, eps, level):
         assert np.array_equal(a, b)
     for a, b in zip(warp[:2], lane[:2]):
         assert np.all(fp64_close(a, b, 1e-13))
+
+
+@pytest.mark.parametrize("eps,pair,u24", host_pairs.AT_BOUNDARY)
+def test_both_forms_decide_alike_at_a_step_boundary(lib, eps, pair, u24):
+    d = dict(host_pairs.BOUNDARY, eps=eps)
+    lane = host_pairs.pairs(lib, d, 6, pair, 1, u24)
+    warp = host_pairs.pairs(lib, d, 6, pair, 1, u24, warp=100)
+    for a, b in zip(warp[2:4], lane[2:4]):
+        assert np.array_equal(a, b)
+    for a, b in zip(warp[:2], lane[:2]):
+        assert np.all(fp64_close(a, b, 1e-13))
