@@ -214,7 +214,7 @@ MLKD_HD Pos operator*(const Pos &a, const Pos &b) { return pos_norm(mul64(a.m, b
 MLKD_HD Pos times(const Pos &a, uint64_t f) { return pos_norm(mul64(a.m, f), a.e); }
 // The bits of the nearest double, for a.e <= 1084 (a number of at least 2^-1021;
 // e = 1086 with m = 2^63 gives 0).  The exponent field of a smaller one wraps:
-// squares and products of draws, which can be below that, go through
+// draws, their products and squares, which can be below that, go through
 // to_double_or_0.
 MLKD_HD uint64_t bits_of(const Pos &a)
 {
@@ -222,7 +222,8 @@ MLKD_HD uint64_t bits_of(const Pos &a)
 }
 MLKD_HD double to_double(const Pos &a) { return from_bits(bits_of(a)); }
 // the same, 0 below 2^-1021
-MLKD_HD double to_double_or_0(const Pos &a) { return from_bits(a.e <= 1084 ? bits_of(a) : 0u); }
+MLKD_HD uint64_t bits_or_0(const Pos &a) { return a.e <= 1084 ? bits_of(a) : 0u; }
+MLKD_HD double to_double_or_0(const Pos &a) { return from_bits(bits_or_0(a)); }
 // a 2^k rounded down, for a 2^k < 2^64
 MLKD_HD uint64_t scaled(const Pos &a, int k)
 {
@@ -377,31 +378,53 @@ MLKD_HD double rsqrt_normal(double x)
 }
 
 // ---------------------------------------------------------------------------
-// cos and sin of 2 pi phase 2^-64: the nearest quarter turn, z in [-pi/4, pi/4]
+// cos and sin of 2 pi phase 2^-64: the nearest quarter turn, z in [-pi/4, pi/4].
+// |z| is formed from the normalised residual, so that sin z keeps its relative
+// precision (2^-61) however small it is; on an axis it is 0 (0 2^-3063).
 // ---------------------------------------------------------------------------
-struct Turn {
-    uint64_t sin, cos;            // magnitudes, in 2^-64 (below 1)
+struct TurnPos {
+    Pos sin, cos;                 // magnitudes
     uint64_t sin_sign, cos_sign;  // the sign bits of doubles
 };
-MLKD_HD Turn sincos_turn(uint64_t phase)
+MLKD_HD TurnPos sincos_pos(uint64_t phase)
 {
     const uint32_t k = (uint32_t)((phase + (1ull << 61)) >> 62);
     const uint64_t r = phase - ((uint64_t)k << 62);           // signed residual
     const bool neg = (int64_t)r < 0;
     const uint64_t a = (neg ? 0u - r : r) << 2;               // |residual| 2^66 <= 2^63
-    const uint64_t z = mul64(a, kTwoPi_61) << 1;              // a 2^-66 2 pi, in 2^-64
+    const int lz = clz64(a | 1u);
+    const uint64_t zn = mul64(a << lz, kTwoPi_61);            // |z| 2^(63 + lz), at least 2^62 (or 0)
+    const uint64_t z = (zn >> lz) << 1;                       // |z| 2^64
     const uint64_t z2 = mul64(z, z);
     const Two p = poly_two<PolySC>(kPolySC, z2);
-    const uint64_t s = z - mul64(z, mul64(z2, p.a));
+    const Pos s = pos_norm(zn - mul64(zn, mul64(z2, p.a)), a ? 63 + lz : 3063);
     const uint64_t c = ~mul64(z2, p.b);                       // cos z >= 0.707
     // sin(z + k pi/2) and cos(z + k pi/2)
     const bool odd = k & 1u;
     const uint64_t sz = neg ? 0x8000000000000000ull : 0u;
-    Turn t;
-    t.sin = odd ? c : s;
-    t.cos = odd ? s : c;
+    TurnPos t;
+    t.sin.m = odd ? c : s.m;
+    t.sin.e = odd ? 64 : s.e;
+    t.cos.m = odd ? s.m : c;
+    t.cos.e = odd ? s.e : 64;
     t.sin_sign = (odd ? 0u : sz) ^ ((uint64_t)(k & 2u) << 62);
     t.cos_sign = (odd ? sz : 0u) ^ ((uint64_t)((k + 1u) & 2u) << 62);
+    return t;
+}
+
+// The same as fractions
+struct Turn {
+    uint64_t sin, cos;            // magnitudes, in 2^-64 (below 1)
+    uint64_t sin_sign, cos_sign;
+};
+MLKD_HD Turn sincos_turn(uint64_t phase)
+{
+    const TurnPos p = sincos_pos(phase);
+    Turn t;
+    t.sin = scaled(p.sin, 64);
+    t.cos = scaled(p.cos, 64);
+    t.sin_sign = p.sin_sign;
+    t.cos_sign = p.cos_sign;
     return t;
 }
 

@@ -106,3 +106,28 @@ def test_both_forms_decide_alike_at_a_step_boundary(lib, eps, pair, u24):
         assert np.array_equal(a, b)
     for a, b in zip(warp[:2], lane[:2]):
         assert np.all(fp64_close(a, b, 1e-13))
+
+
+@pytest.mark.parametrize("B", [53, 24])
+def test_normal_variates_keep_their_relative_precision(lib, B):
+    """nu and chi near every axis, down to the smallest residual of the phase,
+    and on it, where one of them is 0: radius, sine and cosine are right to
+    2^-57 relative, and each product is rounded to FP64 once (0.6 ulp)."""
+    quarter = 1 << (B - 2)
+    off = sorted({0, 1, 2, 3} | {(1 << k) + d for k in range(2, B - 3) for d in (-1, 0, 1)})
+    rng = np.random.default_rng(B)
+    p = np.array([(q * quarter + s * o) % (1 << B) for q in range(4) for o in off for s in (-1, 1)]
+                 + list(rng.integers(0, 1 << B, 4000)), np.uint64)
+    p = np.where(p == 0, np.uint64(1 << B), p)                         # uniforms are 1 to 2^B
+    n = np.stack([rng.integers(1, 1 << (B - 1), len(p)).astype(np.uint64), p, p], axis=1)
+    nu, chi = host_pairs.draws(lib, B, n, 0.5)[:2]
+    r = np.sqrt(-2 * np.log(n[:, 0].astype(LD) / LD(1 << B)))
+    k = (p + np.uint64(quarter // 2)) // np.uint64(quarter)
+    z = (p.astype(np.int64) - k.astype(np.int64) * quarter).astype(LD) * (8 * np.arctan(LD(1))) / LD(1 << B)
+    q = (k & np.uint64(3)).astype(int)
+    for got, exact in ((nu, r * np.choose(q, [np.cos(z), -np.sin(z), -np.cos(z), np.sin(z)])),
+                       (chi, r * np.choose(q, [np.sin(z), np.cos(z), -np.sin(z), -np.cos(z)]))):
+        assert np.all(got[exact == 0] == 0.0)
+        at = exact != 0
+        err = np.abs(got - exact)[at] / np.spacing(np.abs(got[at]))
+        assert np.all(err <= 0.6), float(np.max(err))
