@@ -289,9 +289,10 @@ MLKD_HD Pos steps_left(int steps, uint64_t left)
 // -ln u for the uniform u = n 2^-B, 1 <= n <= 2^B.  n is normalised
 // to x in [1/2, 1); with the reciprocal c of the upper end of x's interval
 // (128 of them), 1 - x c = rho < 2^-7 and -ln x = ln c + rho + rho^2/2 + ...
-// + rho^8/8.  Above 1 - 2^-12 (one draw in 4096), where the logarithm is about
-// the small difference itself, the caller takes log_near_one: it keeps FP64's
-// relative error there.
+// + rho^8/8.  In the last interval below u = 1, where c = 1 and the logarithm
+// is about rho itself, the sum is in units of 2^-71, which holds FP64's
+// precision down to 2^-12.  Above 1 - 2^-12 (one draw in 4096) the caller takes
+// log_near_one.
 // ---------------------------------------------------------------------------
 template <int B, typename Tab> MLKD_HD Pos neg_log(uint64_t n, const Tab &tab)
 {
@@ -302,16 +303,18 @@ template <int B, typename Tab> MLKD_HD Pos neg_log(uint64_t n, const Tab &tab)
     const uint64_t rho = 0u - (((uint64_t)(uint32_t)(x >> 32) * c << 17) + ((uint64_t)(uint32_t)x * c >> 15));
     const uint64_t y = rho << 7;                              // 2^7 rho as a fraction
     const uint32_t yh = (uint32_t)(y >> 32);
-    // 1/4 + rho/5 + rho^2/6 + rho^3/7 + rho^4/8, then 1/3 + rho (.), 1/2 + rho (.)
-    uint32_t t = (1u << 11) / 7u + (yh >> 28);
-    t = (1u << 18) / 6u + umulhi(yh, t);
-    t = (1u << 25) / 5u + umulhi(yh, t);
-    t = (1u << 30) + umulhi(yh, t);
-    const uint64_t s = 0x5555555555555555ull + ((uint64_t)yh * t >> 7);
+    // 1/4 + rho/5 + rho^2/6 + rho^3/7 + rho^4/8 in 2^-33, then 1/3 + rho (.), 1/2 + rho (.)
+    uint32_t t = ((1u << 12) + 3u) / 7u + (yh >> 27);
+    t = ((1u << 19) + 3u) / 6u + umulhi(yh, t);
+    t = ((1u << 26) + 2u) / 5u + umulhi(yh, t);
+    t = (1u << 31) + umulhi(yh, t);
+    const uint64_t s = 0x5555555555555555ull + ((uint64_t)yh * t >> 8);
     const uint64_t w = 0x8000000000000000ull + (mul64(y, s) >> 7);
-    const uint64_t l = tab.ln(j) + rho + (mul64(y, mul64(y, w)) >> 14);
+    const uint64_t yw = mul64(y, w);                          // 2^7 (rho/2 + ...)
     const int k = lz + B - 64;                                // whole powers of two in 1/u
-    return pos_fixed(k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l, k > 0 ? 58 : 64);
+    const bool last = k == 0 && j == 127;
+    const uint64_t l = (last ? y : tab.ln(j) + rho) + (mul64(y, yw) >> (last ? 7 : 14));
+    return pos_fixed(k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l, k > 0 ? 58 : last ? 71 : 64);
 }
 
 // -ln(1 - w) for 0 <= w < 2^-12, in FP64

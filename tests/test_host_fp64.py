@@ -131,3 +131,26 @@ def test_normal_variates_keep_their_relative_precision(lib, B):
         at = exact != 0
         err = np.abs(got - exact)[at] / np.spacing(np.abs(got[at]))
         assert np.all(err <= 0.6), float(np.max(err))
+
+
+@pytest.mark.parametrize("B", [53, 24])
+def test_logarithm_keeps_its_precision_near_one(lib, B):
+    """E = -ln u.  In the last interval, E = rho (1 + rho/2 + ...) < 2^-7.99, the
+    inner sum in 32 bits is off by 2 units of 2^-33 and the step above it drops
+    2^-41: 2^-55.5 of E, 0.18 ulp.  In the next ones sums of at most 3 units of
+    2^-64 and the same of rho^4 at E >= 2^-8: 0.2 ulp.  With one rounding 0.75
+    ulp, and below 2^-12 FP64 with a term of 2^-13 at most: a rounding to nearest.  Every power of two of
+    1 - u and its neighbours, and the ends of the last intervals."""
+    top = 1 << B
+    rng = np.random.default_rng(B)
+    v = {(1 << k) + d for k in range(B - 1) for d in (-1, 0, 1)} | {int(j * top / 256) + d for j in range(1, 5) for d in (-1, 0, 1)}
+    v |= {int(top * 2.0 ** -e) for e in rng.uniform(6, min(40, B - 1), 20000)}
+    n = np.array(sorted(top - u for u in v if 0 <= u < top), np.uint64)
+    E = host_pairs.draws(lib, B, np.stack([n, n, n], axis=1), 0.5)[2]
+    exact = -np.log1p(-((np.uint64(top) - n).astype(LD) / LD(top)))
+    at = exact > 0
+    assert np.all(E[~at] == 0.0)
+    err = ((E - exact)[at] / np.spacing(E[at])).astype(float)
+    assert np.max(np.abs(err)) <= 0.75, np.max(np.abs(err))
+    small = exact[at] < 2.0**-12
+    assert abs(np.mean(err[small])) <= 5 * 0.29 / np.sqrt(np.sum(small)) and np.max(np.abs(err[small])) <= 0.51
