@@ -234,6 +234,13 @@ MLKD_HD uint64_t scaled(const Pos &a, int k)
 // v 2^-sh rounded down, for either sign of sh (sh > -64)
 MLKD_HD uint64_t shift_to(uint64_t v, int sh) { return sh < 0 ? v << -sh : sh < 64 ? v >> sh : 0u; }
 
+// x, or 0 where x is negative
+MLKD_HD double not_negative(double x)
+{
+    const uint64_t b = bits_of(x);
+    return from_bits((int64_t)b < 0 ? 0u : b);
+}
+
 // n as a double, n >= 1
 MLKD_HD double from_u32(uint32_t n)
 {

@@ -224,12 +224,14 @@ __device__ __forceinline__ bool pair_event_fp64(PairState<double> &st, const Lev
             const Background<double>::Unit c = Background<double>::kd_unit<false>(sc, nu2);
             const double chit = fx::bits_of(st.den) ? st.num * A::rsqrt_(st.den) : st.chi_first;   // den >= 0
             st.xc += fma(st.vc, st.oc, fma(c.D, chit, nu * c.om));
-            // the coarse flight ends at the same collision, to_end steps later
+            // the coarse flight ends at the same collision, to_end steps later.  (The whole
+            // steps come from E/(R dt), whose rounding can put to_end R dt above E by an
+            // ulp: nothing in a position, but a length that is read out is not negative.)
             st.oc = to_end > 0 ? fma(-fx::from_u32((uint32_t)to_end), bg.Rdt, E) : E;
             st.whole_c = fl.whole - to_end;
             st.left_c = fl.left;
             if constexpr (!std::is_same<Trace, NoTrace>::value)
-                tr->coarse(nu, st.oc, chit);
+                tr->coarse(nu, fx::not_negative(st.oc), chit);
             st.ic = st.Ec;
             st.vc = nu;
             ++st.evc;

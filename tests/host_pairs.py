@@ -171,3 +171,11 @@ AT_BOUNDARY = [(float.fromhex(e), pair, u24) for e, pair, u24 in (
     ("0x1.5ab3fced1e871p-4", 1, False), ("0x1.ea4fec05af416p-4", 1, False), ("0x1.0608ee7b3f7a3p-3", 5, False),
     ("0x1.c784eeb88ed90p-4", 7, False), ("0x1.5f18e07268fccp-4", 9, False), ("0x1.e40e71800ea5ap-4", 2, True),
     ("0x1.cd1257f72e48cp-4", 4, True), ("0x1.b79b2aeed81c9p-4", 10, True), ("0x1.cc76e56447539p-4", 17, True))]
+
+# (eps, pair, 24-bit stream) of level 2 of FLIGHTS: a fine flight ends at a
+# coarse step's end, and E is below that many times R dt by an ulp
+FLIGHTS = dict(T=1.0, dt0=0.5, M=8, L=2, seed=59, qoi=0, init=0)
+AT_COARSE_END = [(float.fromhex(e), pair, u24) for e, pair, u24 in (
+    ("0x1.7c9c195fd5b89p-3", 4, False), ("0x1.66eea40163041p-3", 6, False), ("0x1.89c447c373d0fp-3", 8, False),
+    ("0x1.8c8140f251fe6p-3", 15, False), ("0x1.47dc91b20357bp-3", 26, False), ("0x1.3a6d4cc372c57p-3", 2, True),
+    ("0x1.5a7f45cc71943p-3", 4, True), ("0x1.16666c0a0a363p-3", 7, True), ("0x1.4bce96d5cd39dp-2", 29, True))]

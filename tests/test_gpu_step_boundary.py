@@ -30,3 +30,15 @@ def test_both_forms_decide_alike(eps, pair, u24):
             assert np.array_equal(a[:32], b)
         for a, b in zip(g[:2], want[:2]):
             assert np.all(fp64_close(a[:32], b, 1e-13))
+
+
+@pytest.mark.parametrize("eps,pair,u24", host_pairs.AT_COARSE_END)
+def test_coarse_flights_are_not_negative(eps, pair, u24):
+    import paper_2004_04071_gb300 as mk
+    p = gpu_problem(mk, dict(host_pairs.FLIGHTS, eps=eps), precision=mk.PREC_FP64_U24 if u24 else mk.PREC_FP64)
+    ctx = mk.Context(0)
+    try:
+        _, E, _, _, taken = ctx.debug_coarse_draws(p, 2, pair, 1, 64)
+    finally:
+        ctx.close()
+    assert len(E) == taken[0] >= 5 and np.all(E >= 0.0)

@@ -154,3 +154,8 @@ def test_logarithm_keeps_its_precision_near_one(lib, B):
     assert np.max(np.abs(err)) <= 0.75, np.max(np.abs(err))
     small = exact[at] < 2.0**-12
     assert abs(np.mean(err[small])) <= 5 * 0.29 / np.sqrt(np.sum(small)) and np.max(np.abs(err[small])) <= 0.51
+
+
+@pytest.mark.parametrize("eps,pair,u24", host_pairs.AT_COARSE_END)
+def test_coarse_flights_are_not_negative(lib, eps, pair, u24):
+    assert host_pairs.pairs(lib, dict(host_pairs.FLIGHTS, eps=eps), 2, pair, 1, u24)[4] >= 0.0
