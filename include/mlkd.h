@@ -314,8 +314,9 @@ MLKD_API mlkd_status mlkd_level_warmup(mlkd_context *ctx, const mlkd_problem *pr
                                        int32_t *tau_out);
 
 /* Validation aid: the KD coefficients of eqs. advection/diffusion and the
- * aggregation quantities of Sec. 3.2 exactly as the pair kernels compute them
- * in `precision` (FP64 state for MLKD_PREC_FP64 and _FP64_U24, FP32 state for
+ * aggregation quantities of Sec. 3.2 exactly as the homogeneous pair kernels compute them
+ * in `precision` (FP64 state for MLKD_PREC_FP64 and _FP64_U24, which holds om,
+ * the square root of beta_hat_sq and d R / sigma; FP32 state for
  * the FP32 modes), for a background (R > 0, mu, sigma >= 0) and n pairs
  * (theta_i, dv_i = v'_i - mu) of device FP64 arrays.  Writes, as FP64 device
  * arrays of n: a, d, hs = h(R theta) = e^{-s} + s - 1, om = 1 - e^{-s} and

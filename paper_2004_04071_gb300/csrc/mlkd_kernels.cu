@@ -569,7 +569,10 @@ cudaError_t launch_coarse_draws(int mode, const PairLaunch &p, int per_pair, dou
 // KD coefficients of eqs. advection/diffusion and the aggregation quantities
 // exactly as the pair kernels compute them in precision Real, for given
 // (theta, v' - mu); the level constants are prepared as for a launch (FP64 on
-// the host, rounded once to Real).
+// the host, rounded once to Real).  In FP64 that is kd_unit, whose results in
+// units of sigma/R are scaled here.  What a pair of a homogeneous background
+// never has (theta < 0, sigma = 0, |v' - mu| beyond 2^400 sigma) takes
+// kd_coeffs, which the heterogeneous FP64 pairs use.
 template <typename Real>
 __global__ void debug_kd_kernel(double R, double mu, double sigma, const double *theta,
                                 const double *dv, unsigned long long n, double *a, double *d,
@@ -584,6 +587,20 @@ __global__ void debug_kd_kernel(double R, double mu, double sigma, const double 
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         Real ai, di, hsi, omi;
+        if constexpr (std::is_same<Real, double>::value) {
+            const double s = R * theta[i], nu = fabs(dv[i]) / sigma;
+            if (Arith<double>::normal_(s) && nu < 0x1p400) {
+                const fx::Pos p = fx::pos_of(nu);
+                const Background<double>::Unit u = Background<double>::kd_unit<true>(fx::pos_of(s), p * p);
+                const double c = sigma / R, c_lo = fma(-c, R, sigma) / R;
+                a[i] = fma(dv[i] * u.om, bg.invR, mu * theta[i]);
+                d[i] = fma(c, u.D, c_lo * u.D);
+                hs[i] = u.hs;
+                om[i] = u.om;
+                bh2[i] = u.beta * u.beta;
+                continue;
+            }
+        }
         bg.kd_coeffs((Real)theta[i], (Real)dv[i], ai, di, hsi, omi);
         a[i] = (double)ai;
         d[i] = (double)di;

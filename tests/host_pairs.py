@@ -29,6 +29,22 @@ extern "C" void draws(int B, const uint64_t *n, const double *s, int64_t count, 
     for (int64_t i = 0; i < count; ++i)
         B == 53 ? draw1<53>(n + 3 * i, s[i], out + 6 * i) : draw1<24>(n + 3 * i, s[i], out + 6 * i);
 }
+// the unit coefficients of phases of length s with normal variates nu
+extern "C" void units(const double *s, const double *nu, int64_t count, double *out)
+{
+    for (int64_t i = 0; i < count; ++i) {
+        const fx::Pos p = fx::pos_of(nu[i]);
+        const Background<double>::Unit u = Background<double>::kd_unit<true>(fx::pos_of(s[i]), p * p);
+        out[4 * i] = u.D, out[4 * i + 1] = u.om, out[4 * i + 2] = u.beta, out[4 * i + 3] = u.hs;
+    }
+}
+// a, d, h(s) and om of kd_coeffs (the heterogeneous pairs) for R = sigma = 1, mu = 0
+extern "C" void het_units(const double *s, const double *nu, int64_t count, double *out)
+{
+    Background<double> bg;
+    bg.R = bg.invR = bg.sigma = 1.0, bg.mu = 0.0, bg.two_c2 = 2.0;
+    for (int64_t i = 0; i < count; ++i) bg.kd_coeffs(s[i], nu[i], out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
+}
 
 struct Least {
     double least = 1.0;
@@ -128,7 +144,7 @@ def build(folder):
                     "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2004_04071_gb300", "csrc"), src,
                     "-o", so], check=True)
     lib = ctypes.CDLL(so)
-    lib.draws.restype = lib.warp_pairs.restype = None
+    lib.draws.restype = lib.warp_pairs.restype = lib.units.restype = lib.het_units.restype = None
     lib.pairs.restype = ctypes.c_double
     return lib
 
@@ -143,6 +159,13 @@ def draws(lib, B, n, s):
     s = np.ascontiguousarray(np.broadcast_to(np.asarray(s, np.float64), len(n)))
     out = np.zeros((len(n), 6))
     lib.draws(B, ptr(n), ptr(s), ctypes.c_int64(len(n)), ptr(out))
+    return out.T
+
+
+def units(lib, s, nu, het=False):
+    """(D, om, beta, h) of kd_unit, or (a, d, h, om) of kd_coeffs."""
+    out = np.zeros((len(s), 4))
+    (lib.het_units if het else lib.units)(ptr(s), ptr(nu), ctypes.c_int64(len(s)), ptr(out))
     return out.T
 
 

@@ -159,3 +159,16 @@ def test_logarithm_keeps_its_precision_near_one(lib, B):
 @pytest.mark.parametrize("eps,pair,u24", host_pairs.AT_COARSE_END)
 def test_coarse_flights_are_not_negative(lib, eps, pair, u24):
     assert host_pairs.pairs(lib, dict(host_pairs.FLIGHTS, eps=eps), 2, pair, 1, u24)[4] >= 0.0
+
+
+def test_coefficients_of_the_heterogeneous_pairs(lib):
+    """kd_coeffs: s < 1 from polynomials (each one rounding, then at most four
+    products and a root: 4 ulp of d, 2 of h and om); beyond, FP64 sums of a
+    few terms, each rounded at its size, at most ten times the sum's."""
+    rng = np.random.default_rng(9)
+    s = np.concatenate([2.0 ** rng.uniform(-40, 0, 4000), rng.uniform(1, 70, 4000), [1.0, np.nextafter(1.0, 0), 44.0, 64.0, 1e6]])
+    nu = np.abs(rng.standard_normal(len(s)))
+    a, d, h, om = host_pairs.units(lib, s, nu, het=True)
+    D, om_x, _ = unit_exact(s, nu)
+    for got, exact, k in ((d, D, 10), (om, om_x, 2), (a, nu * om_x, 3)):
+        assert np.max(np.abs(got - exact) / np.spacing(got)) <= k
