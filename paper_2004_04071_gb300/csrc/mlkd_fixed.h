@@ -201,6 +201,20 @@ MLKD_HD Pos pos_fixed(uint64_t v, int e)                      // v 2^-e, v != 0
     r.e = e + lz;
     return r;
 }
+// the same of v + low 2^-32, for v >= 2^32
+MLKD_HD Pos pos_fixed(uint64_t v, uint32_t low, int e)
+{
+    const int lz = clz64(v) & 31;
+    Pos r;
+#ifdef __CUDA_ARCH__
+    const uint32_t h = __funnelshift_l((uint32_t)v, (uint32_t)(v >> 32), lz), m = __funnelshift_l(low, (uint32_t)v, lz);
+    r.m = (uint64_t)h << 32 | m;
+#else
+    r.m = v << lz | (uint64_t)low << lz >> 32;
+#endif
+    r.e = e + lz;
+    return r;
+}
 MLKD_HD Pos pos_norm(uint64_t p, int e)                       // p 2^-e, p in [2^62, 2^64)
 {
     const int sh = (int)(p >> 63) ^ 1;
@@ -296,10 +310,10 @@ MLKD_HD Pos steps_left(int steps, uint64_t left)
 // -ln u for the uniform u = n 2^-B, 1 <= n <= 2^B.  n is normalised
 // to x in [1/2, 1); with the reciprocal c of the upper end of x's interval
 // (128 of them), 1 - x c = rho < 2^-7 and -ln x = ln c + rho + rho^2/2 + ...
-// + rho^8/8.  In the last interval below u = 1, where c = 1 and the logarithm
-// is about rho itself, the sum is in units of 2^-71, which holds FP64's
-// precision down to 2^-12.  Above 1 - 2^-12 (one draw in 4096) the caller takes
-// log_near_one.
+// + rho^8/8, in units of 2^-64 and 14 bits more of the series.  In the last
+// interval below u = 1, where c = 1, ln c and rho are exact and those bits hold
+// FP64's precision down to 2^-12 (elsewhere they change nothing).  Above
+// 1 - 2^-12 (one draw in 4096) the caller takes log_near_one.
 // ---------------------------------------------------------------------------
 template <int B, typename Tab> MLKD_HD Pos neg_log(uint64_t n, const Tab &tab)
 {
@@ -317,11 +331,10 @@ template <int B, typename Tab> MLKD_HD Pos neg_log(uint64_t n, const Tab &tab)
     t = (1u << 31) + umulhi(yh, t);
     const uint64_t s = 0x5555555555555555ull + ((uint64_t)yh * t >> 8);
     const uint64_t w = 0x8000000000000000ull + (mul64(y, s) >> 7);
-    const uint64_t yw = mul64(y, w);                          // 2^7 (rho/2 + ...)
+    const uint64_t q = mul64(y, mul64(y, w));                 // 2^14 (rho^2/2 + ...)
+    const uint64_t l = tab.ln(j) + rho + (q >> 14);
     const int k = lz + B - 64;                                // whole powers of two in 1/u
-    const bool last = k == 0 && j == 127;
-    const uint64_t l = (last ? y : tab.ln(j) + rho) + (mul64(y, yw) >> (last ? 7 : 14));
-    return pos_fixed(k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l, k > 0 ? 58 : last ? 71 : 64);
+    return pos_fixed(k > 0 ? (l >> 6) + (uint64_t)k * kLn2_58 : l, (uint32_t)q << 18, k > 0 ? 58 : 64);
 }
 
 // -ln(1 - w) for 0 <= w < 2^-12, in FP64
@@ -392,49 +405,74 @@ MLKD_HD double rsqrt_normal(double x)
 // |z| is formed from the normalised residual, so that sin z keeps its relative
 // precision (2^-61) however small it is; on an axis it is 0 (0 2^-3063).
 // ---------------------------------------------------------------------------
+struct Residual {
+    uint64_t a;                   // |phase - k 2^62| 2^2, at most 2^63
+    uint32_t k;                   // quarter turns
+    bool neg;
+};
+MLKD_HD Residual quarter_turns(uint64_t phase)
+{
+    Residual q;
+    q.k = (uint32_t)((phase + (1ull << 61)) >> 62);
+    const uint64_t r = phase - ((uint64_t)q.k << 62);
+    q.neg = (int64_t)r < 0;
+    q.a = (q.neg ? 0u - r : r) << 2;
+    return q;
+}
+// the signs of sin(z + k pi/2) and cos(z + k pi/2)
+MLKD_HD uint64_t sin_sign_of(const Residual &q)
+{
+    return (!(q.k & 1u) && q.neg ? 0x8000000000000000ull : 0u) ^ ((uint64_t)(q.k & 2u) << 62);
+}
+MLKD_HD uint64_t cos_sign_of(const Residual &q)
+{
+    return ((q.k & 1u) && q.neg ? 0x8000000000000000ull : 0u) ^ ((uint64_t)((q.k + 1u) & 2u) << 62);
+}
+
 struct TurnPos {
     Pos sin, cos;                 // magnitudes
     uint64_t sin_sign, cos_sign;  // the sign bits of doubles
 };
 MLKD_HD TurnPos sincos_pos(uint64_t phase)
 {
-    const uint32_t k = (uint32_t)((phase + (1ull << 61)) >> 62);
-    const uint64_t r = phase - ((uint64_t)k << 62);           // signed residual
-    const bool neg = (int64_t)r < 0;
-    const uint64_t a = (neg ? 0u - r : r) << 2;               // |residual| 2^66 <= 2^63
-    const int lz = clz64(a | 1u);
-    const uint64_t zn = mul64(a << lz, kTwoPi_61);            // |z| 2^(63 + lz), at least 2^62 (or 0)
+    const Residual q = quarter_turns(phase);
+    const int lz = clz64(q.a | 1u);
+    const uint64_t zn = mul64(q.a << lz, kTwoPi_61);          // |z| 2^(63 + lz), at least 2^62 (or 0)
     const uint64_t z = (zn >> lz) << 1;                       // |z| 2^64
     const uint64_t z2 = mul64(z, z);
     const Two p = poly_two<PolySC>(kPolySC, z2);
-    const Pos s = pos_norm(zn - mul64(zn, mul64(z2, p.a)), a ? 63 + lz : 3063);
+    const Pos s = pos_norm(zn - mul64(zn, mul64(z2, p.a)), q.a ? 63 + lz : 3063);
     const uint64_t c = ~mul64(z2, p.b);                       // cos z >= 0.707
-    // sin(z + k pi/2) and cos(z + k pi/2)
-    const bool odd = k & 1u;
-    const uint64_t sz = neg ? 0x8000000000000000ull : 0u;
+    const bool odd = q.k & 1u;
     TurnPos t;
     t.sin.m = odd ? c : s.m;
     t.sin.e = odd ? 64 : s.e;
     t.cos.m = odd ? s.m : c;
     t.cos.e = odd ? s.e : 64;
-    t.sin_sign = (odd ? 0u : sz) ^ ((uint64_t)(k & 2u) << 62);
-    t.cos_sign = (odd ? sz : 0u) ^ ((uint64_t)((k + 1u) & 2u) << 62);
+    t.sin_sign = sin_sign_of(q);
+    t.cos_sign = cos_sign_of(q);
     return t;
 }
 
-// The same as fractions
+// The same as fractions, right to 2^-62 absolute
 struct Turn {
     uint64_t sin, cos;            // magnitudes, in 2^-64 (below 1)
     uint64_t sin_sign, cos_sign;
 };
 MLKD_HD Turn sincos_turn(uint64_t phase)
 {
-    const TurnPos p = sincos_pos(phase);
+    const Residual q = quarter_turns(phase);
+    const uint64_t z = mul64(q.a, kTwoPi_61) << 1;
+    const uint64_t z2 = mul64(z, z);
+    const Two p = poly_two<PolySC>(kPolySC, z2);
+    const uint64_t s = z - mul64(z, mul64(z2, p.a));
+    const uint64_t c = ~mul64(z2, p.b);
+    const bool odd = q.k & 1u;
     Turn t;
-    t.sin = scaled(p.sin, 64);
-    t.cos = scaled(p.cos, 64);
-    t.sin_sign = p.sin_sign;
-    t.cos_sign = p.cos_sign;
+    t.sin = odd ? c : s;
+    t.cos = odd ? s : c;
+    t.sin_sign = sin_sign_of(q);
+    t.cos_sign = cos_sign_of(q);
     return t;
 }
 
