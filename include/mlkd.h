@@ -206,7 +206,9 @@ MLKD_API void mlkd_context_destroy(mlkd_context *ctx);
  * (Alg. 1 on level 0, Alg. 2 with the Sec. 3 coupling on level >= 1) on
  * `stream` and returns their sums.  Pair p of level l always uses the Philox
  * stream keyed by (seed, request, l, p), so any split of a pair range gives
- * the same pairs.  hist_out (host, 3*nbins counts or NULL) receives per bin
+ * the same pairs: the same events, and the same positions, in FP64 modes up to
+ * the rounding of their sums (a call of few long pairs adds a pair's increments
+ * in another order than a call of many).  hist_out (host, 3*nbins counts or NULL) receives per bin
  * the number of fine positions, coarse positions, and pairs with both in it.
  * Synchronous: returns after the sums are on the host. */
 MLKD_API mlkd_status mlkd_run_level(mlkd_context *ctx, const mlkd_problem *problem, int level,

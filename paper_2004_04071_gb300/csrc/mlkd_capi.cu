@@ -255,15 +255,18 @@ namespace {
 // One pair per warp (32 of its events per step) instead of one per lane: for
 // coupled homogeneous FP64 pairs, while the chains of the lanes, not the work,
 // set the length of the launch.  A warp's work per pair goes with events + 32 (the
-// start and the last, partial step); the lines cross at 100 to 110 pairs per SM
-// times events / (events + 32) (measured at 2048, 512, 128, 64 and 32 events a
-// pair, one in every step: 16 000, 15 000, 13 500, 11 000, 8000 pairs on 152 SMs; with
-// longer flights later: level 8 at eps = 0.1 19 000).  1000 pairs of level 10 at
-// eps = 1e-3 (2048 events): 4.29 -> 0.39 ms; 100 of level 8 at eps = 0.1: 0.36 -> 0.04;
-// 4000: 0.39 -> 0.11.  Decisions and counts are the same, positions differ by
-// the order of their sums (rms error against extended precision 2e-16 to
-// 3.5e-16 on long pairs, 3e-16 to 1.5e-15 one pair per lane).  FP32 pairs keep the
-// lane form, whose rounding their results carry.
+// start and the last, partial step).  The two forms cross at 160 to 190 pairs per SM
+// times events / (events + 32): at 2048, 512, 128, 64 and 32 events a pair, one in
+// every step, above 28 000 (4.98 ms, 5.28 one pair per lane) and at 27 000, 21 000,
+// 16 000 and 12 500 pairs on 152 SMs; with longer flights later.  The rule stays
+// below that at 100, where the line lay before the warp form took its flights from
+// fixed point: between the two one pair per lane takes up to 1.8 times as long.
+// 1000 pairs of level 10 at eps = 1e-3 (2048 events): 4.48 ms one pair per lane,
+// 0.30 one per warp; 4000 of level 8 at eps = 0.1: 0.39 and 0.09.  Decisions and
+// counts are the same, positions differ by the order of their sums (rms error
+// against extended precision 2e-16 to 3.5e-16 on long pairs, 3e-16 to 1.5e-15 one
+// pair per lane).  FP32 pairs keep the lane form, whose rounding their results
+// carry.
 constexpr double kWarpPairLeast = 32.0;
 constexpr double kWarpPairsPerSm = 100.0;
 

@@ -91,7 +91,8 @@ MLKD_HD uint32_t umulhi(uint32_t a, uint32_t b)
 // a b 2^-64 and a b 2^-32, rounded down, at most two units below.  The high
 // halves of the cross products and one wide product: 8.2 per clock and SM
 // measured, against 6.6 with the carry of the low halves and 6.4 for
-// __umul64hi (2^20 pairs of level 8 of the periodic problem: 11.4 -> 10.0 ms).
+// __umul64hi (2^20 pairs of level 8 of the periodic problem: 8.52, 9.51 and
+// 9.41 ms).
 MLKD_HD uint64_t mul64(uint64_t a, uint64_t b)
 {
     const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
@@ -131,8 +132,8 @@ template <typename P> MLKD_HD uint64_t poly(const uint64_t (&c)[P::kLead][1], ui
 // Two polynomials in the same argument.  The 64-bit steps are a rolled loop
 // over coefficients in constant memory: the FP64 event loop is longer than the
 // instruction caches like (unrolled here too, 2^20 pairs of level 8 of the
-// periodic problem take 13.3 ms, so 11.3 ms; rolled in poly() as well, the deep
-// levels lose 12 %).
+// periodic problem take 10.2 ms, so 8.52 ms; rolled in poly() as well 8.69 ms, and
+// of level 6 at eps = 1e-3 7.95 ms, so 7.07 ms).
 struct Two {
     uint64_t a, b;
 };

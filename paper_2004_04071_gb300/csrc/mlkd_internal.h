@@ -64,8 +64,8 @@ template <typename Real> struct BgParams {
 
 // Idle lanes a warp of the per-level kernel gathers before it takes up new
 // pairs.  Coupled homogeneous pairs, which are started and summed 32 at a time
-// (2^20 pairs of level 8 of the periodic problem): 2 (FP32 1.22 ms, 1.22 with 3,
-// 1.25 with 4, 1.26 with 6, 1.30 with 8; FP64 8.88, 9.00, 9.25, 9.48, 9.87).  The
+// (2^20 pairs of level 8 of the periodic problem): 2 (FP32 1.18 ms, 1.19 with 3,
+// 1.21 with 4, 1.23 with 6, 1.27 with 8; FP64 8.52, 8.61, 8.75, 8.96, 9.33).  The
 // others sum and start them there and then: 6, and 8 for the heterogeneous
 // event, which is longer against a start (4 loses 1 %).
 template <int PHYS, bool COUPLED> constexpr int kRefillMin = PHYS == 1 ? 8 : COUPLED ? 2 : 6;

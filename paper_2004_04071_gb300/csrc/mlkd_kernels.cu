@@ -27,7 +27,7 @@ template <> __device__ __forceinline__ const BgParams<double> &level_params<doub
 // homogeneous background fits 64 registers (8 blocks of 128 threads); the
 // heterogeneous pair state does not, and at 64 registers its kernel kept the
 // FP64 pipe 21-83 % busy (ncu) without a line of FP64 arithmetic, so it gets
-// 128 (4 blocks); the FP64 form is bound by the FP64 pipe.
+// 128 (4 blocks).  FP64 state takes what it needs (118 registers, 4 blocks).
 template <typename Real, int PHYS> struct MinBlocks { static constexpr int value = PHYS == 1 ? 4 : 8; };
 template <int PHYS> struct MinBlocks<double, PHYS> { static constexpr int value = 1; };
 
@@ -39,9 +39,10 @@ template <typename Real> struct PhysState<Real, 1> { typedef HetPairState<Real> 
 // Per warp: pairs started 32 at a time, and a ring of finished pairs that are
 // summed 32 at a time, so that neither path runs for only the few lanes that
 // fell idle together, and lanes wait less.  For coupled homogeneous pairs, with
-// a loop that holds nothing but the event (level 8 of the periodic problem,
-// 2^20 pairs: FP32 1.37 -> 1.20 ms, FP64 9.16 -> 8.54; 1000 pairs of level 10,
-// whose chains are all there is: 1.15 -> 0.86 ms, FP64 4.58 -> 4.30).  Uncoupled
+// a loop that holds nothing but the event (what the two gave when they came in,
+// 2^20 pairs of level 8 of the periodic problem: FP32 1.37 -> 1.20 ms, FP64
+// 9.16 -> 8.54; 1000 FP32 pairs of level 10 at eps = 1e-3, whose chains are all
+// there is: 1.15 -> 0.86 ms).  Uncoupled
 // pairs have so few events that the queues cost more than they save (5e6 paths
 // of level 0: FP32 0.18 ms without, 0.21 with them), and the heterogeneous
 // event is long enough (level 10 of B1: 2.39 and 2.43 ms).
@@ -104,8 +105,9 @@ __device__ __forceinline__ void sum_rows(double *rows, int stride, int count, do
 // Run by the last block of a launch: the summed rows into the launch's sums.
 // Folding this into the pair kernel saves a launch and, in an estimate, the
 // launch that accumulated the histogram, and one copy brings both results
-// to the host: 2000 FP64 pairs with 20 bins 88 -> 78 us, 300 paths with 128 bins
-// 50 -> 41 us, a small adaptive estimate with 64 bins 0.81 -> 0.70 ms.
+// to the host (when it came in: 2000 FP64 pairs with 20 bins 88 -> 78 us, 300
+// paths with 128 bins 50 -> 41 us, a small adaptive estimate with 64 bins
+// 0.81 -> 0.70 ms).
 __device__ __forceinline__ void finish_launch(const PairLaunch &P, const double *w)
 {
     const int t = threadIdx.x;

@@ -176,13 +176,17 @@ __device__ __forceinline__ bool pair_start(PairState<Real> &st, unsigned long lo
 }
 
 // One fine event of the FP64 state; returns true when the pair has reached T.
-// The FP64 pipe bounds it (two operations per clock and SM), so everything
-// that can be is integer: draws, coefficients, weights and flights are
+// With every quantity in FP64 the FP64 pipe bounded it (two operations per
+// clock and SM), so everything that can be is integer: draws, coefficients, weights and flights are
 // positive numbers with 64-bit mantissas (fx::Pos) or fractions, step counts
 // and window tests integers.  What is left in FP64 are the sums: 4 operations
 // for the position and 6 for the window per fine event and 6 per coarse one,
-// against about 45 and 27 with every quantity in FP64 (131 071 pairs of level 8
-// of the periodic problem: 1.54 ms, 1.86 ms with FP64 products).
+// against about 45 and 27 before.  At level 8 of the periodic problem (eps = 0.1)
+// a fine event with its share of a coarse one takes 92 products of fractions
+// and 15 FP64 operations, 11.2 and 8.5 clocks of an SM; 131 071 pairs take
+// 1.29 ms, three times that: the pipes share 54 % of the issue slots, and a
+// warp waits for its own chain of products (profiles/pair_kernel_fp64_periodic.md).
+// FP64 products in place of fx::Pos took 1.86 ms against 1.54 when they went.
 template <int CPL, int RECIPE, typename Trace>
 __device__ __forceinline__ bool pair_event_fp64(PairState<double> &st, const LevelCtx<double> &L,
                                                 const PhiloxKeys &keys, bool coupled_rt, Trace *tr)
