@@ -264,7 +264,7 @@ namespace {
 // 1000 pairs of level 10 at eps = 1e-3 (2048 events): 4.48 ms one pair per lane,
 // 0.30 one per warp; 4000 of level 8 at eps = 0.1: 0.39 and 0.09.  Decisions and
 // counts are the same, positions differ by the order of their sums (rms error
-// against extended precision 2e-16 to 3.5e-16 on long pairs, 3e-16 to 1.5e-15 one
+// against extended precision 1.7e-16 to 3.8e-16 on long pairs, 3e-16 to 1.5e-15 one
 // pair per lane).  FP32 pairs keep the lane form, whose rounding their results
 // carry.
 constexpr double kWarpPairLeast = 32.0;

@@ -131,7 +131,8 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
             Background<double>::kd_unit<true>(fx::pos_of(bg.Rdt) * fx::steps_left(0, left_p), nu2);
         om = f.om;
         bh = f.beta;
-        if (valid) dx = fma(vp, Ep, fma(f.D, chi, dv * om));
+        // D chi is the largest term of a long step: added last, it is rounded once
+        if (valid) dx = fma(f.D, chi, fma(dv, om, vp * Ep));
     } else {
         const Real theta = bg.dt * ((Real)(sq + 1) - qp);      // eq. diffusive-time
         bg.kd_coeffs(theta, dv, a, dd, hs, om);
@@ -226,7 +227,7 @@ __device__ __forceinline__ bool warp_pair_step(PairState<Real> &st, const LevelC
                 if constexpr (kUnit) {
                     const fx::Pos sc = fx::pos_of(bg.Rdt) * fx::steps_left(ecp - ic_pre - wc_pre - 1, left_pre);
                     const Background<double>::Unit c = Background<double>::kd_unit<false>(sc, nu2);
-                    dxc = fma(vc_pre, qc_pre, fma(c.D, chit, dv * c.om));
+                    dxc = fma(c.D, chit, fma(dv, c.om, vc_pre * qc_pre));
                 } else {
                     const Real thc = bg.dt * ((Real)(ecp - ic_pre) - qc_pre);
                     Real hsc;
